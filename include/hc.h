@@ -471,7 +471,7 @@ HC_API int hc_mlp_train_step(hc_mlp* mlp, const float* x_dev, const float* t_dev
  * losses_host[epochs] receives, per epoch, the mean training loss over every
  * 50th minibatch.  feat_dev: n x in float; labels_dev: n uint32.  Set the
  * initial parameters first (hc_mlp_set_params).  Allocates about
- * 50 n + 4 batch (in + 1) bytes of scratch on cuda_stream and returns when
+ * 50 n bytes of scratch on cuda_stream and returns when
  * the training has finished.  HC_ERR_ARG if batch > max_batch or n < batch.
  */
 HC_API int hc_mlp_fit(hc_mlp* mlp, const float* feat_dev, const uint32_t* labels_dev, uint32_t n,
