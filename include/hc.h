@@ -424,9 +424,11 @@ HC_API int hc_features(hc_index* idx, const void* q_dev, uint32_t nq, float* fea
 
 /*
  * hc_probe_labels -- for each query, the minimal p in [0, p_max] whose top-k
- * (ids) equals the top-k at p_max: a per-query binary search, valid because
- * the windows and so the results are nested in p.  p_min_dev: nq uint32.
- * Allocates scratch of about 12*k + 8 bytes per query on cuda_stream.
+ * (ids) equals the top-k at p_max: the depth at which the last of those
+ * neighbours enters a window (the windows, and so the results, are nested in
+ * p).  p_min_dev: nq uint32.  Allocates scratch on cuda_stream for up to
+ * 131,072 queries at a time (fewer when it does not fit): the workspace of
+ * hc_query_ordered and 8*k bytes per query.
  */
 HC_API int hc_probe_labels(hc_index* idx, const void* q_dev, uint32_t nq, uint32_t k,
                            uint32_t p_max, uint32_t* p_min_dev, void* cuda_stream);

@@ -528,10 +528,24 @@ OrderLayout order_layout(const hc_index* idx, uint32_t nq) {
     return L;
 }
 
-// hc_query_ordered's work on a checked workspace of order_layout(idx, nq).bytes:
-// the order keys, their sort, the batch search, then the walk in curve-0 order.
-int enqueue_ordered(hc_index* idx, const void* q_dev, uint32_t nq, uint32_t k, uint32_t p,
-                    int32_t* out_ids_dev, void* out_dist_dev, char* ws, cudaStream_t s) {
+}  // namespace
+
+namespace hc {
+
+size_t ordered_workspace(const hc_index* idx, uint32_t nq) { return order_layout(idx, nq).bytes; }
+
+const uint32_t* ordered_ranks(const hc_index* idx, uint32_t nq, const char* ws) {
+    return reinterpret_cast<const uint32_t*>(ws + order_layout(idx, nq).order);
+}
+
+const uint32_t* ordered_positions(const hc_index* idx, uint32_t nq, const char* ws) {
+    return reinterpret_cast<const uint32_t*>(ws + order_layout(idx, nq).pos);
+}
+
+// hc_query_ordered's work on a checked workspace: the order keys, their sort,
+// the batch search, then the walk in curve-0 order.
+int ordered_query(const hc_index* idx, const void* q_dev, uint32_t nq, uint32_t k, uint32_t p,
+                  int32_t* out_ids_dev, void* out_dist_dev, char* ws, cudaStream_t s) {
     const OrderLayout L = order_layout(idx, nq);
     const uint32_t curves = idx->params.curves;
     uint64_t* keys = reinterpret_cast<uint64_t*>(ws + L.keys);
@@ -568,6 +582,10 @@ int enqueue_ordered(hc_index* idx, const void* q_dev, uint32_t nq, uint32_t k, u
     return status_of(launch_query(v, q_dev, nq, k, p, out_ids_dev, out_dist_dev, s, nullptr,
                                   nullptr, sp.out_ids, pos));
 }
+
+}  // namespace hc
+
+namespace {
 
 // hc_query_host's work: the queries up on cs (into the index's staging), the
 // walk on s behind them (in key order for large batches), the results down
@@ -620,7 +638,7 @@ int enqueue_host_query(hc_index* idx, const void* q_host, uint32_t nq, uint32_t 
         if (landed) cudaEventDestroy(landed);
         if (rc) return rc;
     }
-    rc = ordered ? enqueue_ordered(idx, idx->st_q, nq, k, p, d_ids, d_dist,
+    rc = ordered ? ordered_query(idx, idx->st_q, nq, k, p, d_ids, d_dist,
                                    static_cast<char*>(idx->st_out) + ws_off, s)
                  : status_of(launch_query(view_of(idx), idx->st_q, nq, k, p, d_ids, d_dist, s));
     if (rc) return rc;
@@ -653,7 +671,7 @@ HC_API int hc_query_ordered(hc_index* idx, const void* q_dev, uint32_t nq, uint3
     if (!is_device_ptr(q_dev) || !is_device_ptr(out_ids_dev) || !is_device_ptr(out_dist_dev) ||
         !is_device_ptr(workspace_dev))
         return HC_ERR_ARG;
-    return enqueue_ordered(idx, q_dev, nq, k, p, out_ids_dev, out_dist_dev,
+    return ordered_query(idx, q_dev, nq, k, p, out_ids_dev, out_dist_dev,
                            static_cast<char*>(workspace_dev), static_cast<cudaStream_t>(cuda_stream));
 }
 

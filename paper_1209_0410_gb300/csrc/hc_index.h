@@ -65,6 +65,15 @@ bool index_keeps_lo(const hc_build_params& P);
 // the device arrays of a laid-out index: list offsets and dim map (both
 // uploaded), keys and ids (uninitialised), from the stream-ordered pool on s
 int index_alloc(hc_index* x, cudaStream_t s);
+// A batch answered in key order (hc_query_ordered) on a device workspace of
+// ordered_workspace(x, nq) bytes, 256-byte aligned.  Afterwards the workspace
+// holds the queries' order (rank -> query) and their positions (curve-major
+// rows: entry c * partitions + j of query i for list j * curves + c).
+size_t ordered_workspace(const hc_index* x, uint32_t nq);
+int ordered_query(const hc_index* x, const void* q_dev, uint32_t nq, uint32_t k, uint32_t p,
+                  int32_t* out_ids, void* out_dist, char* workspace, cudaStream_t s);
+const uint32_t* ordered_ranks(const hc_index* x, uint32_t nq, const char* workspace);
+const uint32_t* ordered_positions(const hc_index* x, uint32_t nq, const char* workspace);
 // frees in stream order on s (default: the legacy stream)
 void index_destroy(hc_index* x, cudaStream_t s = cudaStreamLegacy);
 

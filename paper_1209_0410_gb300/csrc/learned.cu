@@ -6,9 +6,8 @@
 //   features   4 per curve: octave encodings of the key gaps to the list
 //              neighbours of the query key, and of the min / mean distance of
 //              the 8 list entries around it (exact, integer-derived values)
-//   labels     minimal p in [0, p_max] whose top-k equals the top-k at p_max,
-//              by a per-query binary search driven by the query kernel
-//              (valid because windows, hence results, are nested in p)
+//   labels     minimal p in [0, p_max] whose top-k equals the top-k at p_max:
+//              the depth at which the last of those neighbours enters a window
 //   model      x^ = (x - mu) * isd;  h1 = relu(x^ W1 + b1);
 //              h2 = relu(h1 W2 + b2);  y = h2 . W3 + b3   (y ~ log2 p)
 //   training   two FP32 kernels per step: the layers forward and back for 32
@@ -784,26 +783,85 @@ __global__ void __launch_bounds__(kPredWarps * 32, 4) predict_depths_kernel(
 }
 
 // ---------------------------------------------------------------- labels
-__global__ void fill_kernel(uint32_t* __restrict__ a, uint32_t v, uint32_t n) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = v;
-}
+// The windows of a query are nested in p, so the top-k at depth p equals the
+// top-k at p_max once every neighbour of the latter lies in some window of depth
+// p: the label is the largest, over those neighbours, of the smallest depth at
+// which any list holds it.  One warp per query (in the batch's key order, whose
+// neighbours share lines of the lists) holds the neighbours in registers, entry
+// r 32 + lane in t[r] of the lane, and streams the ids of its windows past a
+// 2048-bit filter of them; the few ids that pass are compared with all: about
+// ten instructions per 32 ids, no row is read.  50,000 queries at p_max = 512 on
+// 10M rows and 8 lists: 8.1 ms, nearly all of it the one walk at p_max, against
+// 82.6 ms for a binary search over p (eleven walks).
+constexpr int kLabelWarps = 8;
+constexpr uint32_t kLabelSlice = 1u << 17;   // queries labelled at once
+constexpr uint32_t kFilterBits = 2048;
 
-__global__ void label_mid_kernel(const uint32_t* __restrict__ lo, const uint32_t* __restrict__ hi,
-                                 uint32_t* __restrict__ mid, uint32_t nq) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nq) mid[i] = lo[i] < hi[i] ? (lo[i] + hi[i]) / 2 : hi[i];
-}
-
-__global__ void label_update_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ ref,
-                                    uint32_t nq, uint32_t k, uint32_t* __restrict__ lo,
-                                    uint32_t* __restrict__ hi, const uint32_t* __restrict__ mid) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nq || lo[i] >= hi[i]) return;
-    bool same = true;
-    for (uint32_t j = 0; j < k; ++j) same &= ids[(size_t)i * k + j] == ref[(size_t)i * k + j];
-    if (same) hi[i] = mid[i];
-    else lo[i] = mid[i] + 1;
+template <int KR>
+__global__ void __launch_bounds__(kLabelWarps * 32) label_kernel(
+    IndexView ix, uint32_t nq, uint32_t k, uint32_t p_max, const int32_t* __restrict__ ref,
+    const uint32_t* __restrict__ order, const uint32_t* __restrict__ pos_cm,
+    uint32_t* __restrict__ out) {
+    __shared__ uint32_t filters[kLabelWarps][kFilterBits / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t w = blockIdx.x * kLabelWarps + warp;
+    if (w >= nq) return;
+    const uint32_t qi = __ldg(order + w);
+    if (!HC_IN_BOUNDS(kSiteQuery, qi, nq)) return;
+    uint32_t* filter = filters[warp];
+    auto slot = [](uint32_t id) { return (id * 2654435761u) >> 21; };
+    for (uint32_t i = lane; i < kFilterBits / 32; i += 32) filter[i] = 0;
+    __syncwarp();
+    uint32_t t[KR], depth[KR];   // 0xFFFFFFFF: no neighbour (ids are below 2^31)
+#pragma unroll
+    for (int r = 0; r < KR; ++r) {
+        const uint32_t e = r * 32 + lane;
+        t[r] = e < k ? (uint32_t)__ldg(ref + (size_t)qi * k + e) : 0xFFFFFFFFu;
+        depth[r] = t[r] == 0xFFFFFFFFu ? 0u : 0xFFFFFFFFu;
+        if (t[r] != 0xFFFFFFFFu) atomicOr(&filter[slot(t[r]) / 32], 1u << (slot(t[r]) % 32));
+    }
+    __syncwarp();
+    const uint32_t curves = ix.P.curves, parts = ix.lists / curves;
+    for (uint32_t L = 0; L < ix.lists; ++L) {
+        const uint64_t off = ix.list_off[L];
+        const uint32_t n = (uint32_t)(ix.list_off[L + 1] - off);
+        const uint32_t pos =
+            __ldg(pos_cm + (size_t)qi * ix.lists + (L % curves) * parts + L / curves);
+        const uint32_t lo = pos > p_max ? pos - p_max : 0u;
+        const uint32_t hi = (uint64_t)pos + p_max < (uint64_t)n ? pos + p_max : n;
+        if (!HC_IN_BOUNDS(kSiteWindow, hi, (uint64_t)n + 1)) continue;
+        constexpr int U = 4;   // loads in flight
+        for (uint32_t base = lo; base < hi; base += 32 * U) {
+            uint32_t id[U];
+            bool ok[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t e = base + 32 * u + (uint32_t)lane;
+                ok[u] = e < hi;
+                id[u] = ok[u] ? __ldg(ix.ids + off + e) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t s = slot(id[u]);
+                uint32_t hit = __ballot_sync(0xffffffffu, ok[u] && (filter[s / 32] >> (s % 32) & 1u));
+                while (hit) {
+                    const int src = __ffs(hit) - 1;
+                    hit &= hit - 1;
+                    const uint32_t x = __shfl_sync(0xffffffffu, id[u], src);
+                    const uint32_t e = base + 32 * u + (uint32_t)src;
+                    const uint32_t d = e >= pos ? e - pos + 1 : pos - e;
+#pragma unroll
+                    for (int r = 0; r < KR; ++r)
+                        if (t[r] == x) depth[r] = min(depth[r], d);
+                }
+            }
+        }
+    }
+    uint32_t label = 0;
+#pragma unroll
+    for (int r = 0; r < KR; ++r) label = max(label, depth[r]);
+    label = __reduce_max_sync(0xffffffffu, label);
+    if (lane == 0) out[qi] = label;
 }
 
 MlpView view_of_mlp(const hc_mlp* M) {
@@ -960,36 +1018,37 @@ HC_API int hc_probe_labels(hc_index* idx, const void* q_dev, uint32_t nq, uint32
     if (nq == 0) return HC_OK;
     if (!dev_ptr(q_dev) || !dev_ptr(p_min_dev) || ((uintptr_t)q_dev & 15)) return HC_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t res = (size_t)nq * k * 4;
-    const size_t bytes = 3 * res + 2 * (size_t)nq * 4 + 1024;
     if (alloc_should_fail()) return HC_ERR_OOM;
+    // slices of the batch bound the scratch: the key-order workspace, then the
+    // neighbours at p_max (ids and distances); smaller ones when memory is short
+    uint32_t slice = nq < kLabelSlice ? nq : kLabelSlice;
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     char* buf = nullptr;
-    if (cudaMallocAsync((void**)&buf, bytes, s) != cudaSuccess) {
+    size_t ws = 0, res = 0;
+    for (;; slice = (slice + 1) / 2) {
+        ws = al(ordered_workspace(idx, slice));
+        res = al((size_t)slice * k * 4);
+        if (cudaMallocAsync((void**)&buf, ws + 2 * res, s) == cudaSuccess) break;
         cudaGetLastError();
-        return HC_ERR_OOM;
+        if (slice <= 1024) return HC_ERR_OOM;
     }
-    int32_t* ref = reinterpret_cast<int32_t*>(buf);
-    int32_t* ids = reinterpret_cast<int32_t*>(buf + res);
-    void* dist = buf + 2 * res;
-    uint32_t* lo = reinterpret_cast<uint32_t*>(buf + 3 * res);
-    uint32_t* mid = lo + nq;
-    uint32_t* hi = p_min_dev;
+    int32_t* ref = reinterpret_cast<int32_t*>(buf + ws);
     const IndexView ix = view_of(idx);
     int rc = HC_OK;
-    if (launch_query(ix, q_dev, nq, k, p_max, ref, dist, s) != cudaSuccess) rc = HC_ERR_CUDA;
-    if (!rc && (cudaMemsetAsync(lo, 0, (size_t)nq * 4, s) != cudaSuccess)) rc = HC_ERR_CUDA;
-    if (!rc) {
-        fill_kernel<<<(nq + 255) / 256, 256, 0, s>>>(hi, p_max, nq);   // hi = p_max
+    for (uint32_t q0 = 0; !rc && q0 < nq; q0 += slice) {
+        const uint32_t b = nq - q0 < slice ? nq - q0 : slice;
+        const uint8_t* q = static_cast<const uint8_t*>(q_dev) + (size_t)q0 * ix.row_bytes;
+        if ((rc = ordered_query(idx, q, b, k, p_max, ref, buf + ws + res, buf, s))) break;
+        const uint32_t* order = ordered_ranks(idx, b, buf);
+        const uint32_t* pos = ordered_positions(idx, b, buf);
+        const unsigned g = (b + kLabelWarps - 1) / kLabelWarps;
+        if (k <= 32)
+            label_kernel<1><<<g, kLabelWarps * 32, 0, s>>>(ix, b, k, p_max, ref, order, pos,
+                                                           p_min_dev + q0);
+        else
+            label_kernel<4><<<g, kLabelWarps * 32, 0, s>>>(ix, b, k, p_max, ref, order, pos,
+                                                           p_min_dev + q0);
         count_launches(1);
-    }
-    uint32_t iters = 1;
-    while ((1u << iters) <= p_max + 1) ++iters;
-    for (uint32_t it = 0; !rc && it <= iters; ++it) {
-        const unsigned g = (nq + 255) / 256;
-        label_mid_kernel<<<g, 256, 0, s>>>(lo, hi, mid, nq);
-        if (launch_query(ix, q_dev, nq, k, 0, ids, dist, s, mid) != cudaSuccess) rc = HC_ERR_CUDA;
-        label_update_kernel<<<g, 256, 0, s>>>(ids, ref, nq, k, lo, hi, mid);
-        count_launches(2);
         if (cudaGetLastError() != cudaSuccess) rc = HC_ERR_CUDA;
     }
     cudaFreeAsync(buf, s);
