@@ -119,46 +119,6 @@ __device__ __forceinline__ uint4 three_halves(float x, float y, float z) {
                       *reinterpret_cast<const uint32_t*>(&b), 0u, 0u);
 }
 
-// Bitonic compare-exchange steps over 32 KR entries, entry r 32 + lane in v[r]
-// of the lane.  merge_sorted: the last phase alone (a bitonic sequence in,
-// ascending out); sort_all: any order in.
-template <int KR>
-__device__ __forceinline__ void bitonic_phase(uint64_t (&v)[KR], int size, int stride, int lane) {
-    if (stride >= 32) {
-        const int rs = stride / 32;
-#pragma unroll
-        for (int r = 0; r < KR; ++r) {
-            if ((r & rs) == 0) {
-                const bool up = ((r * 32) & size) == 0;   // size > 32 here
-                const uint64_t lo = min(v[r], v[r | rs]), hi = max(v[r], v[r | rs]);
-                v[r] = up ? lo : hi;
-                v[r | rs] = up ? hi : lo;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < KR; ++r) {
-            const uint64_t o = __shfl_xor_sync(0xffffffffu, v[r], stride);
-            const bool up = ((r * 32 + lane) & size) == 0, first = (lane & stride) == 0;
-            v[r] = (first == up) ? min(v[r], o) : max(v[r], o);
-        }
-    }
-}
-template <int KR>
-__device__ __forceinline__ void merge_sorted(uint64_t (&v)[KR], int lane) {
-#pragma unroll
-    for (int stride = 16 * KR; stride >= 1; stride >>= 1)
-        bitonic_phase<KR>(v, 64 * KR, stride, lane);
-}
-template <int KR>
-__device__ __forceinline__ void sort_all(uint64_t (&v)[KR], int lane) {
-#pragma unroll
-    for (int size = 2; size <= 32 * KR; size <<= 1)
-#pragma unroll
-        for (int stride = size / 2; stride >= 1; stride >>= 1)
-            bitonic_phase<KR>(v, size, stride, lane);
-}
-
 // A query's list of KS slots: the best k in order, then `pending` appended
 // ones.  The whole warp sorts it; returns the k-th entry.
 template <int KS>

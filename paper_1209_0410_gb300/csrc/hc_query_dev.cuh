@@ -1,7 +1,6 @@
 // Device helpers of the query path shared by the query kernel, the exact
 // brute force and the depth predictor: 16-byte row gathers, exact distances,
-// the reduce-scatter of per-lane partial sums, and lower_bound on 128-bit
-// keys.
+// the walks of a query's windows, and lower_bound on 128-bit keys.
 #pragma once
 
 #include <type_traits>
@@ -43,23 +42,6 @@ __device__ __forceinline__ float acc_vec(uint4 a, uint4 b, float acc) {
 
 __device__ __forceinline__ uint32_t dist_bits(uint32_t d) { return d; }
 __device__ __forceinline__ uint32_t dist_bits(float d) { return __float_as_uint(d); }
-
-// v[j] = this lane's partial of sub-batch j (j < LPR).  Returns the full sum of
-// sub-batch (lane % LPR) over the LPR lanes of the lane's group.
-template <int LPR, typename Acc>
-__device__ __forceinline__ Acc reduce_scatter(Acc (&v)[LPR], uint32_t s) {
-#pragma unroll
-    for (int w = LPR / 2; w >= 1; w >>= 1) {
-        const bool upper = (s & (uint32_t)w) != 0;
-#pragma unroll
-        for (int t = 0; t < w; ++t) {
-            const Acc send = upper ? v[t] : v[t + w];
-            const Acc keep = upper ? v[t + w] : v[t];
-            v[t] = keep + __shfl_xor_sync(0xffffffffu, send, w);
-        }
-    }
-    return v[0];
-}
 
 // Candidates produced per lane by one 32-row chunk: rows wider than 8 lanes
 // are reduced 8 sub-batches at a time, leaving one candidate per group.
@@ -403,50 +385,13 @@ __device__ __forceinline__ void load_positions(const IndexView& ix, const uint8_
     }
 }
 
-// Algorithm 2 for one query over the lists L0, L0 + Lstep, ... into the
-// warp's running top-k: keys, positions, then every window in 32-entry steps
-// (the next step's ids are loaded while the current rows are in flight).
-template <bool F32, int LPR, int KR>
-__device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t* qrow,
-                                             uint32_t depth, uint32_t k, uint32_t L0,
-                                             uint32_t Lstep, uint32_t* pos_w, WarpTopK<KR>& top,
-                                             int lane, const int64_t* pos_in = nullptr,
-                                             const uint32_t* pos_cm = nullptr) {
-    load_positions(ix, qrow, pos_w, lane, L0, Lstep, pos_in, pos_cm);
-    const uint32_t s = (uint32_t)lane % LPR;
-    const uint4 qv0 = s < (ix.row_bytes >> 4) ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
-    const uint8_t* db = static_cast<const uint8_t*>(ix.db);
-    for (uint32_t L = L0; L < ix.lists; L += Lstep) {
-        const uint64_t off = ix.list_off[L];
-        const uint32_t n = (uint32_t)(ix.list_off[L + 1] - off);
-        const uint32_t pos = pos_w[L];
-        const uint32_t lo = pos > depth ? pos - depth : 0u;
-        const uint32_t hi = (uint64_t)pos + depth < (uint64_t)n ? pos + depth : n;
-        if (!HC_IN_BOUNDS(kSiteWindow, hi, (uint64_t)n + 1)) continue;
-        const uint32_t* idl = ix.ids + off;
-        uint32_t next = lo + (uint32_t)lane < hi ? __ldg(idl + lo + lane) : 0u;
-        for (uint32_t base = lo; base < hi; base += 32) {
-            const uint32_t id = HC_IN_BOUNDS(kSiteRow, next, ix.rows) ? next : 0u;
-            const uint32_t cnt = min(32u, hi - base);
-            if (base + 32 < hi)
-                next = base + 32 + (uint32_t)lane < hi ? __ldg(idl + base + 32 + lane) : 0u;
-            uint64_t cand[ChunkWidth<LPR>::NG];
-            chunk_candidates_n<F32, LPR>(db, ix.row_bytes, qrow, qv0, id, cnt, lane, cand);
-#pragma unroll
-            for (int c = 0; c < ChunkWidth<LPR>::NG; ++c) top.offer(cand[c], k, lane);
-        }
-    }
-}
-
-
 // ---------------------------------------------------------------------------
-// Staged form of the window walk for rows of at most 128 bytes (one 16-byte
-// vector per lane of a row group, LPR <= 8): the windows of all lists are
-// packed back to back and walked in steps of 32 entries (a step may span
-// several short windows, so short or uneven windows fill whole steps); the
-// rows of the next step are copied into a per-warp shared-memory ring with
+// Staged form of the window walk for rows of at most 128 bytes: the windows of
+// all lists are packed back to back and walked in steps of 32 entries (a step
+// may span several short windows, so short or uneven windows fill whole steps);
+// the rows of the next step are copied into a per-warp shared-memory ring with
 // cp.async (no registers held while they are in flight) while the current
-// step's rows are reduced, and the step after that has its ids loaded.
+// step's rows are reduced, a row per lane.
 // Waits are the hardware's cp.async group waits.
 __device__ __forceinline__ void cp_async16(uint32_t saddr, const void* g) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(g) : "memory");
@@ -498,126 +443,394 @@ __device__ __forceinline__ uint32_t pack_windows(const IndexView& ix, uint32_t d
     return carry;
 }
 
-// ids of packed step s (entries 32 s .. 32 s + 31 of the concatenated
-// windows): lane l finds its window by binary search over win_pre
-__device__ __forceinline__ uint32_t packed_ids(const IndexView& ix, const uint32_t* win_at,
-                                               const uint32_t* win_pre, uint32_t nm,
-                                               uint32_t total, uint32_t s, int lane) {
-    const uint32_t e = 32 * s + (uint32_t)lane;
-    if (e >= total) return 0u;
-    uint32_t lo = 0, count = nm;   // largest m with win_pre[m] <= e
-    while (count > 1) {
-        const uint32_t half = count >> 1;
-        if (win_pre[lo + half] <= e) {
-            lo += half;
-            count -= half;
+// A lane's place in the packed windows: the window of its last entry, the
+// packed entry at which that window ends, and first entry - packed entry of it.
+// A lane's entries only grow, so most calls find the window they left.
+struct WindowCursor {
+    uint32_t m = ~0u, end = 0, base = 0;
+
+    // id of packed entry e, or of the last one (total - 1) when e is past it; e
+    // is not below the lane's last one, total > 0
+    __device__ __forceinline__ uint32_t id(const IndexView& ix, const uint32_t* win_at,
+                                           const uint32_t* win_pre, uint32_t nm, uint32_t total,
+                                           uint32_t e) {
+        e = min(e, total - 1);
+        while (e >= end) {
+            ++m;
+            end = m + 1 < nm ? win_pre[m + 1] : total;
+            base = win_at[m] - win_pre[m];
+        }
+        const uint32_t ent = base + e;
+        if (!HC_IN_BOUNDS(kSiteEntry, ent, ix.list_off[ix.lists])) return 0u;
+        const uint32_t id = __ldg(ix.ids + ent);
+        return HC_IN_BOUNDS(kSiteRow, id, ix.rows) ? id : 0u;
+    }
+
+    // the window of packed entry e, so that a walk starting there need not pass
+    // all before it (the largest window that starts at or before e)
+    __device__ __forceinline__ void seek(const uint32_t* win_pre, uint32_t nm, uint32_t e) {
+        uint32_t lo = 0, count = nm;
+        while (count > 1) {
+            const uint32_t half = count >> 1;
+            if (win_pre[lo + half] <= e) {
+                lo += half;
+                count -= half;
+            } else {
+                count = half;
+            }
+        }
+        m = lo - 1;
+    }
+};
+
+// Rows of at most 128 bytes staged in shared memory, 32 to a stage: row r's
+// 16-byte vector c lies at vector c ^ f(r) of the row, so that eight lanes
+// reading vector c of eight neighbouring rows touch eight different bank groups
+// (f(r) = the row's low bits, as many as the row's vector count has factors of
+// two, taken from bit 3 - that many up).
+struct RowSwizzle {
+    uint32_t shift, mask;
+    __device__ __forceinline__ explicit RowSwizzle(uint32_t vecs) {
+        const uint32_t g = vecs & (0u - vecs);   // a power of two, at most 8
+        mask = g - 1;
+        shift = 3u - (uint32_t)(31 - __clz(g));
+    }
+    __device__ __forceinline__ uint32_t at(uint32_t r, uint32_t c) const {
+        return c ^ ((r >> shift) & mask);
+    }
+};
+
+// The two-stage pipeline of staged rows: while the copies of one step are in
+// flight the step before it is reduced, a whole row per lane, so no partial sums
+// cross lanes.  FULL: rows of exactly 16 LPR bytes (128 or 64).  add() takes the
+// next step's ids (lane l: row l; the rows of lanes at or past cnt are copied but
+// not offered), finish() reduces the last one.  ring: two stages of 32 rows,
+// 128-byte aligned.  START: the first step's candidates are sorted into the list
+// instead of inserted one by one (a call in the loop: where registers are short
+// its spills cost more than the insertions).
+constexpr uint32_t kRingRows = 64;     // two stages of 32 rows
+constexpr uint32_t kWideRing = 8192;   // bytes: two stages of walk_wide
+
+template <bool F32, int LPR, int KR, bool FULL, bool START>
+struct StagedSteps {
+    const uint8_t* db;               // (values: a reference would put them in local memory)
+    uint32_t row_bytes;
+    uint8_t* ring;
+    uint4 q[8];                      // the query's vectors (zero past the row)
+    uint32_t id = 0, cnt = 0;        // of the step in flight (cnt = 0: none)
+    uint32_t at = 0;                 // byte offset of its stage
+    RowSwizzle sw;
+    uint64_t thr;                    // the k-th candidate so far
+    bool fresh;                      // no candidate so far
+
+    __device__ __forceinline__ StagedSteps(const IndexView& ix, const uint8_t* qrow,
+                                           uint8_t* ring_mem, const WarpTopK<KR>& top, uint32_t k)
+        : db(static_cast<const uint8_t*>(ix.db)),
+          row_bytes(ix.row_bytes),
+          ring(ring_mem),
+          sw(ix.row_bytes >> 4),
+          thr(top.kth(k)) {
+        fresh = START && __all_sync(0xffffffffu, top.v[0] == kEmpty);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            q[c] = c < LPR && (FULL || (uint32_t)c < (row_bytes >> 4)) ? ldg16(qrow + c * 16)
+                                                                       : make_uint4(0, 0, 0, 0);
+    }
+
+    __device__ __forceinline__ uint32_t other_stage() const {
+        return (FULL ? 512u * LPR : 32u * row_bytes) - at;
+    }
+
+    // copies of one step: lane (c = lane % LPR, g = lane / LPR) moves vector c of
+    // rows g, g + 32 / LPR, ... (vectors past the row are skipped)
+    __device__ __forceinline__ void issue(uint32_t nid, uint32_t stage, int lane) {
+        constexpr uint32_t RPI = 32 / LPR;
+        const uint32_t c = (uint32_t)lane % LPR, g = (uint32_t)lane / LPR;
+        const uint8_t* col = db + c * 16;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring) + stage;
+        if constexpr (FULL) {
+            // 8 vectors: rows g + 4 t swap by g or g + 4; 4 vectors: rows g + 8 t by g / 2
+            const uint32_t x = LPR == 8 ? c ^ g : c ^ ((g >> 1) & 3u);
+            const uint32_t even = base + g * (16 * LPR) + x * 16;
+            const uint32_t odd = LPR == 8 ? even ^ 64u : even;
+#pragma unroll
+            for (int t = 0; t < LPR; ++t) {
+                const uint32_t rid = __shfl_sync(0xffffffffu, nid, (int)(g + RPI * (uint32_t)t));
+                cp_async16((t & 1 ? odd : even) + 512u * (uint32_t)t,
+                           col + (uint64_t)rid * (16u * LPR));
+            }
         } else {
-            count = half;
+            const bool colok = c < (row_bytes >> 4);
+#pragma unroll
+            for (int t = 0; t < LPR; ++t) {
+                const uint32_t r = g + RPI * (uint32_t)t;
+                const uint32_t rid = __shfl_sync(0xffffffffu, nid, (int)r);
+                if (colok)
+                    cp_async16(base + r * row_bytes + sw.at(r, c) * 16,
+                               col + (size_t)rid * row_bytes);
+            }
         }
     }
-    const uint64_t ent = (uint64_t)win_at[lo] + (e - win_pre[lo]);
-    if (!HC_IN_BOUNDS(kSiteEntry, ent, ix.list_off[ix.lists])) return 0u;
-    const uint32_t id = __ldg(ix.ids + ent);
-    return HC_IN_BOUNDS(kSiteRow, id, ix.rows) ? id : 0u;
-}
 
-// copies of one step: lane (c = lane % 8, g = lane / 8) moves vector c of
-// rows g, g + 4, ..., g + 28 (rows past cnt and vectors past the row are
-// skipped)
-__device__ __forceinline__ void issue_step(const uint8_t* __restrict__ db, uint32_t row_bytes,
-                                           uint32_t sbuf, uint32_t id, uint32_t cnt, int lane) {
-    const uint32_t c = (uint32_t)lane & 7u, g = (uint32_t)lane >> 3;
-    const bool colok = c < (row_bytes >> 4);
+    // Distance of the staged row `lane` to the query.  float32: a sum per
+    // vector, then the vectors' sums by halves of LPR (v and v + LPR / 2, then
+    // LPR / 4, ...), the order in which rows read by LPR lanes are reduced.
+    __device__ __forceinline__ uint32_t distance(int lane) const {
+        const uint32_t vecs = FULL ? (uint32_t)LPR : row_bytes >> 4;
+        const uint8_t* row = ring + at + (uint32_t)lane * (FULL ? 16u * LPR : row_bytes);
+        const uint32_t x = (LPR == 8 && FULL) ? (uint32_t)lane & 7u
+                           : FULL             ? ((uint32_t)lane >> 1) & 3u
+                                              : sw.at((uint32_t)lane, 0);
+        auto vec = [&](int c) {
+            return *reinterpret_cast<const uint4*>(row + (((uint32_t)c ^ x) << 4));
+        };
+        if constexpr (F32) {
+            float part[LPR];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const uint32_t r = g + 4u * (uint32_t)t;
-        const uint32_t rid = __shfl_sync(0xffffffffu, id, (int)r);
-        if (colok && r < cnt)
-            cp_async16(sbuf + r * row_bytes + c * 16, db + (size_t)rid * row_bytes + c * 16);
+            for (int c = 0; c < LPR; ++c)
+                part[c] = (uint32_t)c < vecs ? acc_vec(vec(c), q[c], 0.f) : 0.f;
+#pragma unroll
+            for (int w = LPR / 2; w >= 1; w >>= 1)
+#pragma unroll
+                for (int c = 0; c < w; ++c) part[c] = part[c] + part[c + w];
+            return __float_as_uint(part[0]);
+        } else {
+            uint32_t acc[2] = {0, 0};
+#pragma unroll
+            for (int c = 0; c < LPR; ++c)
+                if ((uint32_t)c < vecs) acc[c & 1] = acc_vec(vec(c), q[c], acc[c & 1]);
+            return acc[0] + acc[1];
+        }
     }
+
+    __device__ __forceinline__ void reduce(WarpTopK<KR>& top, uint32_t k, int lane) {
+        __syncwarp();   // every lane's copies have landed
+        const uint32_t d = distance(lane);
+        const bool live = (uint32_t)lane < cnt;
+        if (START && fresh) {
+            fresh = false;
+            if (top.start(live ? ((uint64_t)d << 32) | id : kEmpty, lane)) {
+                thr = top.kth(k);
+                return;
+            }
+        }
+        top.offer_row(d, id, live, k, thr, lane);
+    }
+
+    __device__ __forceinline__ void add(uint32_t nid, uint32_t ncnt, WarpTopK<KR>& top, uint32_t k,
+                                        int lane) {
+        __syncwarp();   // every lane is done with the stage before it is refilled
+        issue(nid, other_stage(), lane);
+        cp_async_commit();
+        if (cnt) {
+            cp_async_wait<1>();
+            reduce(top, k, lane);
+        }
+        id = nid;
+        cnt = ncnt;
+        at = other_stage();
+    }
+    __device__ __forceinline__ void finish(WarpTopK<KR>& top, uint32_t k, int lane) {
+        cp_async_wait<0>();
+        if (cnt) reduce(top, k, lane);
+        cnt = 0;
+    }
+};
+
+// The walk of a query's packed windows (rows of at most 128 bytes): steps
+// part, part + parts, ... of 32 entries, the ids of the next two on their way.
+template <bool F32, int LPR, int KR, bool FULL, bool SPLIT, bool START>
+__device__ __forceinline__ void walk_staged(const IndexView& ix, const uint8_t* qrow, uint32_t k,
+                                            const uint32_t* win_at, const uint32_t* win_pre,
+                                            uint32_t nm, uint32_t total, uint32_t my_part,
+                                            uint32_t my_parts, uint8_t* ring, WarpTopK<KR>& top,
+                                            int lane) {
+    const uint32_t part = SPLIT ? my_part : 0u, parts = SPLIT ? my_parts : 1u;
+    const uint32_t steps = total / 32 + (total % 32 != 0);
+    if (part >= steps) return;
+    StagedSteps<F32, LPR, KR, FULL, START> pipe(ix, qrow, ring, top, k);
+    WindowCursor cur;
+    const uint32_t stride = 32 * parts;
+    uint32_t e = 32 * part + (uint32_t)lane;
+    if (part) cur.seek(win_pre, nm, e);
+    auto id_of = [&](uint32_t step, uint32_t at) {
+        return step < steps ? cur.id(ix, win_at, win_pre, nm, total, at) : 0u;
+    };
+    uint32_t id0 = id_of(part, e), id1 = id_of(part + parts, e + stride);
+    for (uint32_t s = part; s < steps; s += parts) {
+        const uint32_t id2 = id_of(s + 2 * parts, e + 2 * stride);
+        pipe.add(id0, min(32u, total - 32 * s), top, k, lane);
+        e += stride;
+        id0 = id1;
+        id1 = id2;
+    }
+    pipe.finish(top, k, lane);
 }
 
-// chunk_candidates_n over rows staged in shared memory (LPR <= 8, so one
-// candidate per lane)
-template <bool F32, int LPR>
-__device__ __forceinline__ uint64_t staged_candidates(const uint8_t* sbuf, uint32_t row_bytes,
-                                                      uint4 qv0, uint32_t id, uint32_t cnt,
-                                                      int lane) {
-    static_assert(LPR <= 8, "staged rows are read one vector per lane");
+// The same for wider rows, LPR lanes to a row: window by window in steps of 32
+// entries, the next step's ids on their way.  A step's rows are read in units of
+// eight 16-byte vectors per lane (vector s + v LPR of eight sub-batches of 32 /
+// LPR rows), each unit copied into one of two 4 KB stages while the unit before
+// it is added up; a lane reads back only what it copied itself.  A unit's sums
+// are those of chunk_candidates_n, reduced in the same order.  Of every `parts`
+// steps in a row this warp takes one.
+template <bool F32, int LPR, int KR, bool SPLIT>
+__device__ __forceinline__ void walk_wide(const IndexView& ix, const uint8_t* qrow, uint32_t k,
+                                          const uint32_t* win_at, const uint32_t* win_pre,
+                                          uint32_t nm, uint32_t total, uint32_t my_part,
+                                          uint32_t my_parts, uint8_t* ring, WarpTopK<KR>& top,
+                                          int lane) {
     using Acc = typename std::conditional<F32, float, uint32_t>::type;
-    constexpr int RPI = 32 / LPR;
+    constexpr uint32_t RPI = 32 / LPR;
+    constexpr int G = 8, NG = LPR / G, COPIES = LPR / G;
+    const uint32_t stride = SPLIT ? 32 * my_parts : 32u;
     const uint32_t s = (uint32_t)lane % LPR, g = (uint32_t)lane / LPR;
-    const bool colok = s < (row_bytes >> 4);
-    Acc part[LPR];
+    const uint32_t row_bytes = ix.row_bytes, vecs = row_bytes >> 4;
+    const uint32_t vpl = (vecs + LPR - 1) / LPR;
+    const uint8_t* db = static_cast<const uint8_t*>(ix.db);
+    const uint4 qv0 = s < vecs ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
+    const uint32_t slot = (uint32_t)__cvta_generic_to_shared(ring) + (uint32_t)lane * 16;
+
+    // steps: entries base .. of the window that ends at hi; m: the window after it
+    uint32_t m = 0, base = 0, hi = 0, skip = SPLIT ? my_part : 0u;
+    auto next_step = [&](uint32_t& id, uint32_t& cnt) {   // cnt = 0: no more
+        if (hi - base > stride) {
+            base += stride;
+        } else {
+            base = hi;
+            while (base == hi && m < nm) {
+                base = win_at[m];
+                const uint32_t len = (m + 1 < nm ? win_pre[m + 1] : total) - win_pre[m];
+                hi = base + len;
+                ++m;
+                if (SPLIT) {
+                    const uint32_t steps = len / 32 + (len % 32 != 0);
+                    if (skip >= steps) {
+                        skip -= steps;
+                        base = hi;
+                    } else {
+                        base += 32 * skip;
+                        skip += my_parts * ((steps - skip + my_parts - 1) / my_parts) - steps;
+                    }
+                }
+            }
+        }
+        cnt = min(32u, hi - base);
+        id = 0;
+        if ((uint32_t)lane < cnt &&
+            HC_IN_BOUNDS(kSiteEntry, base + (uint32_t)lane, ix.list_off[ix.lists]))
+            id = __ldg(ix.ids + base + lane);
+        if (!HC_IN_BOUNDS(kSiteRow, id, ix.rows)) id = 0;
+    };
+    auto issue = [&](uint32_t id, uint32_t cnt, uint32_t gi, uint32_t v, uint32_t stage) {
+        const uint32_t col = s + v * LPR;
+        const uint8_t* at = db + col * 16;
+        const uint32_t to = slot + stage * 4096;
 #pragma unroll
-    for (int j = 0; j < LPR; ++j) {
-        const uint32_t r = (uint32_t)j * RPI + g;
-        const uint4 rv = colok ? *reinterpret_cast<const uint4*>(sbuf + r * row_bytes + s * 16)
-                               : make_uint4(0, 0, 0, 0);
-        part[j] = acc_vec(rv, qv0, Acc(0));
+        for (int j = 0; j < G; ++j) {
+            const uint32_t r = (gi * G + (uint32_t)j) * RPI + g;
+            const uint32_t rid = __shfl_sync(0xffffffffu, id, (int)r);
+            if (r < cnt && col < vecs) cp_async16(to + 512u * (uint32_t)j, at + (size_t)rid * row_bytes);
+        }
+    };
+    uint32_t id, cnt, nid, ncnt, stage = 0;
+    next_step(id, cnt);
+    if (cnt == 0) return;
+    issue(id, cnt, 0, 0, 0);
+    cp_async_commit();
+    next_step(nid, ncnt);
+    while (cnt) {
+        uint32_t fid = 0, fcnt = 0;
+        if (ncnt) next_step(fid, fcnt);
+#pragma unroll 1
+        for (uint32_t gi = 0; gi < (uint32_t)NG; ++gi) {
+            Acc part[G];
+#pragma unroll
+            for (int j = 0; j < G; ++j) part[j] = Acc(0);
+#pragma unroll 1
+            for (uint32_t v = 0; v < vpl; ++v) {
+                // the unit after this one: this row part, this step or the next
+                const bool same = v + 1 < vpl, step = !same && gi + 1 == (uint32_t)NG;
+                issue(step ? nid : id, step ? ncnt : cnt, same ? gi : (step ? 0u : gi + 1),
+                      same ? v + 1 : 0u, stage ^ 1u);
+                cp_async_commit();
+                const uint32_t col = s + v * LPR;
+                const bool colok = col < vecs;
+                const uint4 qv =
+                    v == 0 ? qv0 : (colok ? ldg16(qrow + col * 16) : make_uint4(0, 0, 0, 0));
+                cp_async_wait<1>();
+                const uint8_t* from = ring + stage * 4096 + lane * 16;
+#pragma unroll
+                for (int j = 0; j < G; ++j) {
+                    uint4 rv = *reinterpret_cast<const uint4*>(from + 512 * j);
+                    if (!colok) rv = make_uint4(0, 0, 0, 0);
+                    part[j] = acc_vec(rv, qv, part[j]);
+                }
+                stage ^= 1u;
+            }
+            // halving steps over the top log2(G) bits of s, then plain sums
+#pragma unroll
+            for (int w = LPR / 2, half = G / 2; half >= 1; w >>= 1, half >>= 1) {
+                const bool upper = (s & (uint32_t)w) != 0;
+#pragma unroll
+                for (int t = 0; t < half; ++t) {
+                    const Acc send = upper ? part[t] : part[t + half];
+                    const Acc keep = upper ? part[t + half] : part[t];
+                    part[t] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+                }
+            }
+            Acc dsum = part[0];
+#pragma unroll
+            for (int w = COPIES / 2; w >= 1; w >>= 1)
+                dsum += __shfl_xor_sync(0xffffffffu, dsum, w);
+            const uint32_t r = (gi * G + s / COPIES) * RPI + g;
+            const uint32_t cid = __shfl_sync(0xffffffffu, id, (int)r);
+            top.offer(r < cnt && (s % COPIES) == 0 ? ((uint64_t)dist_bits(dsum) << 32) | cid
+                                                   : kEmpty,
+                      k, lane);
+        }
+        id = nid, cnt = ncnt;
+        nid = fid, ncnt = fcnt;
     }
-    const Acc dsum = reduce_scatter<LPR>(part, s);
-    const uint32_t r = s * RPI + g;
-    const uint32_t cid = __shfl_sync(0xffffffffu, id, (int)r);
-    return r < cnt ? ((uint64_t)dist_bits(dsum) << 32) | cid : kEmpty;
+    cp_async_wait<0>();
 }
 
-// S ring stages: the copies of S - 1 steps are in flight while one is
-// reduced, and the ids of the step after those are loaded.
-template <bool F32, int LPR, int KR, int S = 2>
-__device__ __forceinline__ void search_lists_staged(const IndexView& ix, const uint8_t* qrow,
-                                                    uint32_t depth, uint32_t k, uint32_t L0,
-                                                    uint32_t Lstep, uint32_t* pos_w,
-                                                    uint32_t* win_pre, uint8_t* ring,
-                                                    WarpTopK<KR>& top, int lane,
-                                                    const int64_t* pos_in = nullptr,
-                                                    const uint32_t* pos_cm = nullptr) {
-    static_assert(S >= 2, "one step reduced while another is in flight");
+// ring: kRingRows rows of the warp's shared memory (rows of at most 128 bytes) or
+// kWideRing bytes; SPLIT: steps part, part + parts, ... only; START as in StagedSteps
+template <bool F32, int LPR, int KR, bool SPLIT, bool START>
+__device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* qrow, uint32_t k,
+                                            const uint32_t* win_at, const uint32_t* win_pre,
+                                            uint32_t nm, uint32_t total, uint32_t part,
+                                            uint32_t parts, uint8_t* ring, WarpTopK<KR>& top,
+                                            int lane) {
+    if constexpr (LPR > 8) {
+        walk_wide<F32, LPR, KR, SPLIT>(ix, qrow, k, win_at, win_pre, nm, total, part, parts, ring,
+                                       top, lane);
+    } else if (ix.row_bytes == 16 * LPR) {
+        walk_staged<F32, LPR, KR, true, SPLIT, START>(ix, qrow, k, win_at, win_pre, nm, total,
+                                                      part, parts, ring, top, lane);
+    } else {
+        walk_staged<F32, LPR, KR, false, SPLIT, START>(ix, qrow, k, win_at, win_pre, nm, total,
+                                                       part, parts, ring, top, lane);
+    }
+}
+
+// Algorithm 2 for one query over the lists L0, L0 + Lstep, ... into the warp's
+// running top-k: positions, packed windows, then their walk.  pos_w, win_pre:
+// one word per list of the index.
+template <bool F32, int LPR, int KR, bool START = false>
+__device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t* qrow,
+                                             uint32_t depth, uint32_t k, uint32_t L0,
+                                             uint32_t Lstep, uint32_t* pos_w, uint32_t* win_pre,
+                                             uint8_t* ring, WarpTopK<KR>& top, int lane,
+                                             const int64_t* pos_in = nullptr,
+                                             const uint32_t* pos_cm = nullptr) {
     load_positions(ix, qrow, pos_w, lane, L0, Lstep, pos_in, pos_cm);
-    const uint32_t s = (uint32_t)lane % LPR;
-    const uint4 qv0 = s < (ix.row_bytes >> 4) ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
-    const uint8_t* db = static_cast<const uint8_t*>(ix.db);
-    const uint32_t row_bytes = ix.row_bytes;
-    const uint32_t stage_bytes = 32 * row_bytes;
-    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     const uint32_t nm = ix.lists > L0 ? (ix.lists - L0 + Lstep - 1) / Lstep : 0;
     uint32_t* win_at = pos_w;   // positions are consumed by pack_windows
     const uint32_t total = pack_windows(ix, depth, L0, Lstep, pos_w, win_at, win_pre, lane);
-    const uint32_t steps = (total + 31) / 32;
-    if (steps == 0) return;
-    // ids[j]: this lane's id of step a + j; steps a .. a + S - 2 are in flight
-    uint32_t ids[S];
-#pragma unroll
-    for (int j = 0; j < S; ++j)
-        ids[j] = (uint32_t)j < steps ? packed_ids(ix, win_at, win_pre, nm, total, j, lane) : 0u;
-#pragma unroll
-    for (int j = 0; j < S - 1; ++j) {
-        if ((uint32_t)j < steps)
-            issue_step(db, row_bytes, ring_s + (uint32_t)j * stage_bytes, ids[j],
-                       min(32u, total - 32 * (uint32_t)j), lane);
-        cp_async_commit();
-    }
-    uint32_t st = 0;   // stage of step a
-    for (uint32_t a = 0; a < steps; ++a) {
-        const uint32_t sn = st == 0 ? S - 1 : st - 1;   // stage of step a + S - 1
-        if (a + S - 1 < steps)
-            issue_step(db, row_bytes, ring_s + sn * stage_bytes, ids[S - 1],
-                       min(32u, total - 32 * (a + S - 1)), lane);
-        cp_async_commit();
-        const uint32_t nid = a + S < steps ? packed_ids(ix, win_at, win_pre, nm, total, a + S, lane)
-                                           : 0u;
-        cp_async_wait<S - 1>();   // step a has landed
-        __syncwarp();
-        top.offer(staged_candidates<F32, LPR>(ring + st * stage_bytes, row_bytes, qv0, ids[0],
-                                              min(32u, total - 32 * a), lane),
-                  k, lane);
-        __syncwarp();             // every lane is done with stage st before it is refilled
-#pragma unroll
-        for (int j = 0; j < S - 1; ++j) ids[j] = ids[j + 1];
-        ids[S - 1] = nid;
-        st = st + 1 == S ? 0u : st + 1;
-    }
-    cp_async_wait<0>();
+    walk_packed<F32, LPR, KR, false, START>(ix, qrow, k, win_at, win_pre, nm, total, 0, 1, ring,
+                                            top, lane);
 }
 
 }  // namespace hc

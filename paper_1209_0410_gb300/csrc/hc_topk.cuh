@@ -22,6 +22,53 @@ namespace hc {
 
 constexpr uint64_t kEmpty = ~0ull;
 
+// Bitonic compare-exchange steps over 32 KR entries, entry r 32 + lane in v[r]
+// of the lane.  merge_sorted: the last phase alone (a bitonic sequence in,
+// ascending out); sort_all: any order in.
+template <int KR>
+__device__ __forceinline__ void bitonic_phase(uint64_t (&v)[KR], int size, int stride, int lane) {
+    if (stride >= 32) {
+        const int rs = stride / 32;
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            if ((r & rs) == 0) {
+                const bool up = ((r * 32) & size) == 0;   // size > 32 here
+                const uint64_t lo = min(v[r], v[r | rs]), hi = max(v[r], v[r | rs]);
+                v[r] = up ? lo : hi;
+                v[r | rs] = up ? hi : lo;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            const uint64_t o = __shfl_xor_sync(0xffffffffu, v[r], stride);
+            const bool up = ((r * 32 + lane) & size) == 0, first = (lane & stride) == 0;
+            v[r] = (first == up) ? min(v[r], o) : max(v[r], o);
+        }
+    }
+}
+template <int KR>
+__device__ __forceinline__ void merge_sorted(uint64_t (&v)[KR], int lane) {
+#pragma unroll
+    for (int stride = 16 * KR; stride >= 1; stride >>= 1)
+        bitonic_phase<KR>(v, 64 * KR, stride, lane);
+}
+template <int KR>
+__device__ __forceinline__ void sort_all(uint64_t (&v)[KR], int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32 * KR; size <<= 1)
+#pragma unroll
+        for (int stride = size / 2; stride >= 1; stride >>= 1)
+            bitonic_phase<KR>(v, size, stride, lane);
+}
+
+// the warp's 32 values in order (out of line: one copy per translation unit)
+static __device__ __noinline__ uint64_t sort_warp(uint64_t x, int lane) {
+    uint64_t v[1] = {x};
+    sort_all<1>(v, lane);
+    return v[0];
+}
+
 template <int KR>
 struct WarpTopK {
     uint64_t v[KR];
@@ -73,6 +120,44 @@ struct WarpTopK {
                 insert(y, lane);
                 thr = kth(k);
             }
+        }
+    }
+
+    // one of 32 candidates as the very first: the list is the sorted candidates;
+    // false (nothing done) when two of them are equal
+    __device__ __forceinline__ bool start(uint64_t cand, int lane) {
+        const uint64_t x = sort_warp(cand, lane);
+        const uint64_t up = __shfl_up_sync(0xffffffffu, x, 1);
+        if (__any_sync(0xffffffffu, lane > 0 && up == x && x != kEmpty)) return false;
+        v[0] = x;
+        return true;
+    }
+
+    // offer one row per lane: distance bits and id (live: the lane has one); thr:
+    // the k-th element, kept by the caller.  The first test is on the distance
+    // bits alone.
+    __device__ __forceinline__ void offer_row(uint32_t dist, uint32_t id, bool live, uint32_t k,
+                                              uint64_t& thr, int lane) {
+        uint32_t m = __ballot_sync(0xffffffffu, live && dist <= (uint32_t)(thr >> 32));
+        while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            const uint64_t y = ((uint64_t)__shfl_sync(0xffffffffu, dist, src) << 32) |
+                               __shfl_sync(0xffffffffu, id, src);
+            if (y < thr) {
+                insert(y, lane);
+                thr = kth(k);
+            }
+        }
+    }
+
+    // a list that store() wrote earlier
+    __device__ __forceinline__ void load(uint32_t k, int lane, const int32_t* ids,
+                                         const uint32_t* dist) {
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            const uint32_t e = (uint32_t)r * 32 + lane;
+            v[r] = e < k && ids[e] >= 0 ? ((uint64_t)dist[e] << 32) | (uint32_t)ids[e] : kEmpty;
         }
     }
 

@@ -40,7 +40,8 @@ struct MultiTask {
 
 constexpr int kMaxWarps = 16;
 constexpr uint32_t kMaxLists = 256;
-constexpr size_t kRingBytes = 64 * 128;   // two 32-row steps of rows up to 128 bytes
+constexpr size_t kRingBytes = kWideRing;   // also kRingRows rows of at most 128 bytes
+static_assert(kRingBytes >= kRingRows * 128, "a ring for rows of either kind");
 
 // Instantiations inside the persistent kernel: row classes uint8 with 4, 8 or
 // 16 lanes per row (wider uint8 rows take 16 lanes and loop), float32 with 16
@@ -60,8 +61,7 @@ uint32_t variant_of(hc_dtype t, uint32_t row_bytes, uint32_t k) {
 // merge; templated on the job's variant.
 // group_buf: 4 x 32 slots per warp of the query's group (warp `sub` owns
 // group_buf + sub * 128).
-// ring: the warp's two-step row ring (64 x 128 bytes) when the plan has
-// rows of at most 128 bytes, else null.
+// ring: the warp's row ring (kRingBytes).
 template <bool F32, int LPR, int KR>
 __device__ void multi_query(const MultiJob& J, uint32_t qi, bool active, uint32_t sub,
                             uint32_t* pos_w, uint32_t lists_cap, uint64_t* group_buf,
@@ -71,16 +71,8 @@ __device__ void multi_query(const MultiJob& J, uint32_t qi, bool active, uint32_
     if (active && !HC_IN_BOUNDS(kSiteMultiQuery, qi, J.nq)) active = false;
     if (active) {
         const uint8_t* qrow = J.q + (size_t)qi * J.ix.row_bytes;
-        if constexpr (LPR <= 8) {
-            if (ring && J.ix.row_bytes <= 128) {
-                search_lists_staged<F32, LPR, KR>(J.ix, qrow, J.p, J.k, sub, J.wpq, pos_w,
-                                                  pos_w + lists_cap, ring, top, lane);
-            } else {
-                search_lists<F32, LPR, KR>(J.ix, qrow, J.p, J.k, sub, J.wpq, pos_w, top, lane);
-            }
-        } else {
-            search_lists<F32, LPR, KR>(J.ix, qrow, J.p, J.k, sub, J.wpq, pos_w, top, lane);
-        }
+        search_lists<F32, LPR, KR>(J.ix, qrow, J.p, J.k, sub, J.wpq, pos_w, pos_w + lists_cap,
+                                   ring, top, lane);
     }
     // one warp per query (the same for every warp of the block: one job per
     // task): the warp's list is the query's, written without a block barrier
@@ -120,15 +112,15 @@ __device__ __forceinline__ void run_variant(const MultiJob& J, uint32_t qi, bool
 
 __global__ void __launch_bounds__(kMaxWarps * 32)
     multi_kernel(const MultiJob* __restrict__ jobs, const MultiTask* __restrict__ tasks,
-                 uint32_t ntasks, uint32_t tile, uint32_t* __restrict__ counter, bool staged,
+                 uint32_t ntasks, uint32_t tile, uint32_t* __restrict__ counter,
                  uint32_t lists_cap) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const uint32_t nwarps = blockDim.x >> 5;
-    uint64_t* merge = reinterpret_cast<uint64_t*>(smem_raw);             // nwarps x 4 x 32
+    uint8_t* rings = smem_raw;                                           // nwarps x kRingBytes
+    uint64_t* merge = reinterpret_cast<uint64_t*>(smem_raw + nwarps * kRingBytes);   // nwarps x 4 x 32
     // per warp: lists_cap positions, then lists_cap window prefixes (lists_cap:
-    // the plan's largest index, a multiple of 4, so the rings stay 16-byte aligned)
+    // the plan's largest index)
     uint32_t* pos = reinterpret_cast<uint32_t*>(merge + nwarps * 4 * 32);
-    uint8_t* rings = reinterpret_cast<uint8_t*>(pos + nwarps * 2 * lists_cap); // nwarps x kRingBytes
     __shared__ uint32_t s_task;
     const int lane = threadIdx.x & 31;
     const uint32_t warp = threadIdx.x >> 5;
@@ -149,7 +141,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
             const bool active = group < per_pass && qo < T.cnt;
             const uint32_t qi = T.q0 + qo;
             uint32_t* pw = pos + (size_t)warp * 2 * lists_cap;
-            uint8_t* ring = staged ? rings + (size_t)warp * kRingBytes : nullptr;
+            uint8_t* ring = rings + (size_t)warp * kRingBytes;
             switch (J.variant) {
 #define HC_V(n) \
     case n: run_variant<n>(J, qi, active, sub, pw, lists_cap, mb, ring, lane); break;
@@ -165,9 +157,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
 
 __global__ void reset_counter_kernel(uint32_t* c) { *c = 0; }
 
-size_t multi_smem(uint32_t nwarps, bool staged, uint32_t lists_cap) {
+size_t multi_smem(uint32_t nwarps, uint32_t lists_cap) {
     return (size_t)nwarps * 4 * 32 * sizeof(uint64_t) +
-           (size_t)nwarps * 2 * lists_cap * sizeof(uint32_t) + (staged ? nwarps * kRingBytes : 0);
+           (size_t)nwarps * 2 * lists_cap * sizeof(uint32_t) + nwarps * kRingBytes;
 }
 
 }  // namespace
@@ -180,7 +172,6 @@ struct hc_multi_plan {
     uint32_t* counter = nullptr;
     unsigned grid = 0;
     size_t smem = 0;
-    bool staged = false;   // some job has rows of at most 128 bytes and <= 8 lanes per row
     uint32_t lists_cap = 4;   // largest number of lists of a job's index, rounded up to 4
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -201,7 +192,7 @@ bool on_device(const void* p) {
 int enqueue(hc_multi_plan* P, cudaStream_t s) {
     reset_counter_kernel<<<1, 1, 0, s>>>(P->counter);
     multi_kernel<<<P->grid, P->cfg.warps_per_block * 32, P->smem, s>>>(
-        P->jobs_dev, P->tasks_dev, P->ntasks, P->cfg.tile, P->counter, P->staged, P->lists_cap);
+        P->jobs_dev, P->tasks_dev, P->ntasks, P->cfg.tile, P->counter, P->lists_cap);
     count_launches(2);
     return cudaGetLastError() == cudaSuccess ? HC_OK : HC_ERR_CUDA;
 }
@@ -301,11 +292,8 @@ HC_API int hc_multi_plan_create(const hc_multi_job* jobs, uint32_t njobs,
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    for (const MultiJob& j : hj) {
-        P->staged |= j.variant / 2 <= 1;   // uint8 rows <= 128 bytes
-        P->lists_cap = std::max(P->lists_cap, (j.ix.lists + 3u) & ~3u);
-    }
-    P->smem = multi_smem(cfg.warps_per_block, P->staged, P->lists_cap);
+    for (const MultiJob& j : hj) P->lists_cap = std::max(P->lists_cap, (j.ix.lists + 3u) & ~3u);
+    P->smem = multi_smem(cfg.warps_per_block, P->lists_cap);
     if (cudaFuncSetAttribute(multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)P->smem) != cudaSuccess) {
         free_plan(P);

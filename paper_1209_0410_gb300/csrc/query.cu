@@ -12,61 +12,35 @@
 //       (order_keys_kernel: every curve's key of every query; a sort by each
 //       curve's key; batch_positions_kernel: a warp per 32 neighbouring keys
 //       of one curve), and the walk reads the positions;
-//   K4  the windows [max(0,pos-p), min(n,pos+p)) are walked 32 entries at a
-//       time: the 32 ids are one load, then each row is read as 16-byte
-//       vectors by LPR lanes (LPR = 8 for 128-byte uint8 rows: four rows per
-//       warp instruction).  Rows of at most 128 bytes are staged: all windows
-//       of the query are packed back to back (a step may span several), and
-//       the next step's rows are copied into a two-step per-warp shared-
-//       memory ring with cp.async while the current step is reduced, so the
-//       bytes in flight are bounded by shared memory instead of registers;
-//       wider rows are gathered into registers, eight 16-byte loads in flight
-//       per lane.  uint8 partial distances use
-//       vabsdiffu4 + dp4a (exact in 32-bit integers), float32 use fma;
-//       a reduce-scatter over the LPR lanes leaves lane l with the distance
-//       of one row of the 32 (LPR-1 shuffles for LPR partial sums);
+//   K4  the windows [max(0,pos-p), min(n,pos+p)) are packed back to back and
+//       walked 32 entries at a time (a step may span several).  Rows of at most
+//       128 bytes are staged: the next step's rows are copied into a two-step
+//       per-warp shared-memory ring with cp.async while the current step is
+//       reduced, so the bytes in flight are bounded by shared memory instead of
+//       registers, and each lane then reads a whole row (16-byte vectors laid
+//       out so that no two lanes of a quarter-warp meet in a bank): no partial
+//       sums cross lanes.  Wider rows are gathered into registers, LPR lanes to
+//       a row and eight 16-byte loads in flight per lane, and reduce-scattered
+//       over the LPR lanes.  uint8 distances use vabsdiffu4 + dp4a (exact in
+//       32-bit integers), float32 use fma;
 //   K5/K6 the 32 packed (distance, id) candidates are offered to one running
 //       warp top-k for the whole query, which drops duplicate ids: the union
 //       over curves and partitions and the Aggregator's reduction in one.
 // The path is a gather bounded by HBM bandwidth; no tensor cores are used.
 #include <algorithm>
 
-#include "hc_dispatch.cuh"
-#include "hc_internal.h"
-#include "hc_query_dev.cuh"
-#include "hc_topk.cuh"
+#include "hc_walk.cuh"
 
 namespace hc {
 
 namespace {
 
-constexpr int kQWarps = 8;
-constexpr int kStages = 2;   // ring stages per warp (deeper rings measured slower)
-
-struct QueryArgs {
-    IndexView ix;
-    const void* q;
-    uint32_t nq, k, p;
-    int32_t* out_ids;
-    void* out_dist;
-    int64_t* out_pos;            // positions-only kernel
-    const uint32_t* p_query;     // per-query depth (overrides p), or null
-    const int64_t* pos_in;       // precomputed lower_bound positions (nq x lists), or null
-    const uint32_t* order;       // warp w answers query order[w], or null (w itself)
-    const uint32_t* pos_cm;      // positions of the batch pass (curve-major rows), or null
-};
-
-#ifndef HC_QUERY_MIN_BLOCKS
-#define HC_QUERY_MIN_BLOCKS 3    // resident blocks per SM the query kernel is compiled for
-                                 // (3 x 8 warps: best at p = 128 and 512 on GB300)
-#endif
-
-// STAGED: rows of at most 128 bytes go through a two-step cp.async ring in
-// shared memory (kQWarps x 2 x 32 rows after the positions and the window
-// prefixes)
-template <bool F32, int LPR, int KR, bool STAGED>
-__global__ void __launch_bounds__(kQWarps * 32, HC_QUERY_MIN_BLOCKS) query_kernel(QueryArgs a) {
-    extern __shared__ __align__(16) uint32_t s_pos[];  // kQWarps x lists, then the rings
+// Rows of at most 128 bytes go through a two-step cp.async ring in shared
+// memory: the block's rings, then its positions and window prefixes.
+// BLOCKS: blocks resident per SM (registers)
+template <bool F32, int LPR, int KR, int BLOCKS>
+__global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t w = blockIdx.x * kQWarps + warp;
     if (w >= a.nq) return;
@@ -75,22 +49,14 @@ __global__ void __launch_bounds__(kQWarps * 32, HC_QUERY_MIN_BLOCKS) query_kerne
     const IndexView& ix = a.ix;
     const uint8_t* qrow = static_cast<const uint8_t*>(a.q) + (size_t)qi * ix.row_bytes;
     const uint32_t depth = a.p_query ? __ldg(a.p_query + qi) : a.p;
+    const uint32_t rb = ring_bytes<LPR>(ix.row_bytes);
+    uint32_t* pos_w = reinterpret_cast<uint32_t*>(smem + kQWarps * rb) + warp * 2 * ix.lists;
     WarpTopK<KR> top;
     top.init();
-    if constexpr (STAGED) {
-        // after the positions: kQWarps x lists window prefixes, then the rings
-        uint32_t* s_pre = s_pos + kQWarps * ix.lists;
-        uint8_t* ring = reinterpret_cast<uint8_t*>(s_pre + kQWarps * ix.lists) +
-                        (size_t)warp * kStages * 32 * ix.row_bytes;
-        search_lists_staged<F32, LPR, KR, kStages>(
-            ix, qrow, depth, a.k, 0, 1, s_pos + warp * ix.lists, s_pre + warp * ix.lists, ring,
-            top, lane, a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
-            a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
-    } else {
-        search_lists<F32, LPR, KR>(ix, qrow, depth, a.k, 0, 1, s_pos + warp * ix.lists, top,
-                                   lane, a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
-                                   a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
-    }
+    search_lists<F32, LPR, KR, BLOCKS == 2>(
+        ix, qrow, depth, a.k, 0, 1, pos_w, pos_w + ix.lists, smem + warp * rb, top, lane,
+        a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
+        a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
     top.template store<F32>(a.k, lane, a.out_ids + (size_t)qi * a.k,
                             static_cast<uint32_t*>(a.out_dist) + (size_t)qi * a.k);
 }
@@ -274,28 +240,20 @@ __global__ void __launch_bounds__(256) fence_kernel(const uint64_t* __restrict__
 
 template <bool F32, int LPR, int KR>
 struct QueryLaunch {
-    template <bool STAGED>
-    static cudaError_t go(const QueryArgs& a, size_t smem, cudaStream_t s) {
+    template <typename K>
+    static cudaError_t go(K kernel, const QueryArgs& a, size_t smem, cudaStream_t s) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
         const unsigned blocks = (unsigned)(((uint64_t)a.nq + kQWarps - 1) / kQWarps);
-        if (STAGED) {
-            cudaError_t e = cudaFuncSetAttribute(query_kernel<F32, LPR, KR, STAGED>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        query_kernel<F32, LPR, KR, STAGED><<<blocks, kQWarps * 32, smem, s>>>(a);
+        kernel<<<blocks, kQWarps * 32, smem, s>>>(a);
         count_launches(1);
         return cudaGetLastError();
     }
     static cudaError_t run(const QueryArgs& a, cudaStream_t s) {
-        const size_t pos_bytes = sizeof(uint32_t) * kQWarps * a.ix.lists;
-        // rows of at most 128 bytes (all rows of 4 or 8 lanes) are staged
-        if constexpr (LPR <= 8) {
-            const size_t smem = 2 * pos_bytes + (size_t)kQWarps * kStages * 32 * a.ix.row_bytes;
-            return go<true>(a, smem, s);
-        } else {
-            return go<false>(a, pos_bytes, s);
-        }
+        const size_t smem =
+            kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 2 * sizeof(uint32_t) * a.ix.lists);
+        return go(query_kernel<F32, LPR, KR, 3>, a, smem, s);
     }
 };
 
