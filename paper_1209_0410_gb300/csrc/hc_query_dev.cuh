@@ -363,6 +363,77 @@ __device__ __forceinline__ void query_positions(const IndexView& ix, const uint8
     __syncwarp();
 }
 
+// query_positions with the lanes of the warp spread over the searches: `each`
+// lanes (a power of two) take one list and probe `each` points of its bracket at
+// once, so a list of n entries takes log(n) / log(each + 1) rounds of one load
+// instead of log2(n).  For few lists per warp.
+__device__ __forceinline__ void query_positions_spread(const IndexView& ix, const uint8_t* qrow,
+                                                       uint32_t* pos_w, int lane, uint32_t L0,
+                                                       uint32_t Lstep) {
+    const uint32_t curves = ix.P.curves;
+    uint64_t khi = 0, klo = 0;
+    if ((uint32_t)lane < curves) curve_key_call(qrow, ix.P, (uint32_t)lane, khi, klo);
+    const uint32_t mine = ix.lists > L0 ? (ix.lists - L0 + Lstep - 1) / Lstep : 0;
+    uint32_t each = 32;
+    while (each > 4 && 32 / each < mine) each /= 2;
+    const uint32_t i = (uint32_t)lane % each, g = (uint32_t)lane / each;
+    const uint32_t group = each == 32 ? 0xFFFFFFFFu : (1u << each) - 1u;
+    for (uint32_t b = 0; b < mine; b += 32 / each) {
+        const uint32_t t = b + g;
+        const bool on = t < mine;
+        const uint32_t L = on ? L0 + t * Lstep : L0;
+        const uint64_t kh = __shfl_sync(0xffffffffu, khi, (int)(L % curves));
+        const uint64_t kl = __shfl_sync(0xffffffffu, klo, (int)(L % curves));
+        const uint64_t off = ix.list_off[L], end = on ? ix.list_off[L + 1] : off;
+        // first point in [first, first + count) where below() no longer holds
+        auto search = [&](uint64_t first, uint64_t count, auto&& below) {
+            while (__any_sync(0xffffffffu, count > 0)) {
+                const bool last = count <= each;
+                const uint64_t at = last ? i : count * (i + 1) / (each + 1);
+                const bool in = at < count;
+                const bool yes = in && below(first + at);
+                const uint32_t n =
+                    (uint32_t)__popc(__ballot_sync(0xffffffffu, yes) >> (g * each) & group);
+                if (last) {
+                    first += n;
+                    count = 0;
+                } else {
+                    const uint64_t lo = n ? count * n / (each + 1) + 1 : 0;
+                    const uint64_t hi = n < each ? count * (n + 1) / (each + 1) : count;
+                    first += lo;
+                    count = hi - lo;
+                }
+            }
+            return first;
+        };
+        uint64_t lo = off, hi = end;
+        if (ix.fence) {
+            // as lower_bound_key: the fence words bracket the answer
+            const uint64_t ja = (off + 15) >> kFenceShift, jb = (end + 15) >> kFenceShift;
+            const uint64_t pk = kh & kFenceMask;
+            auto word = [&](uint64_t j) {
+                return HC_IN_BOUNDS(kSiteSearch, j, ix.fence_len) ? __ldg(ix.fence + j) : ~0ull;
+            };
+            const uint64_t jl = search(ja, jb > ja ? jb - ja : 0, [&](uint64_t j) {
+                return word(j) < pk;
+            });
+            const bool tie = jl < jb && word(jl) == pk;
+            const uint64_t ju = search(tie ? jl + 1 : jl, tie ? jb - jl - 1 : 0, [&](uint64_t j) {
+                return word(j) <= pk;
+            });
+            if (jl > ja) lo = ((jl - 1) << kFenceShift) + 1;
+            if (ju < jb) hi = ju << kFenceShift;
+        }
+        const uint64_t pos = search(lo, hi > lo ? hi - lo : 0, [&](uint64_t e) {
+            if (!HC_IN_BOUNDS(kSiteSearch, e, end)) return false;
+            const uint64_t h = __ldg(ix.keys_hi + e);
+            return h < kh || (h == kh && entry_key_lo(ix, L, e) < kl);
+        });
+        if (on && i == 0) pos_w[L] = (uint32_t)(pos - off);
+    }
+    __syncwarp();
+}
+
 // The query's positions in lists L0, L0 + Lstep, ... into pos_w[L]: read
 // from a batch pass when one ran (pos_in: list order, int64; pos_cm: curve-
 // major uint32, entry c * partitions + j for list j * curves + c), else

@@ -181,4 +181,44 @@ struct WarpTopK {
     }
 };
 
+// Sorted list `other` into sorted list `mine`, both 32 KR words of shared memory
+// with distinct elements each, by one warp: the k smallest distinct of the two
+// lead `mine` afterwards.  With k <= 16 KR the smaller of element e of one and
+// 32 KR - 1 - e of the other are a bitonic sequence of the 32 KR smallest, which
+// hold k distinct ones; otherwise `other` is offered to `mine`.  Out of line.
+template <int KR>
+static __device__ __noinline__ void merge_lists(uint64_t* mine, const uint64_t* other, uint32_t k,
+                                                int lane) {
+    WarpTopK<KR> top;
+#pragma unroll
+    for (int r = 0; r < KR; ++r) top.v[r] = mine[r * 32 + lane];
+    if (k > 16 * KR) {
+#pragma unroll 1
+        for (int r = 0; r < KR; ++r) top.offer(other[r * 32 + lane], k, lane);
+    } else {
+#pragma unroll
+        for (int r = 0; r < KR; ++r)
+            top.v[r] = min(top.v[r], other[32 * KR - 1 - (r * 32 + lane)]);
+        merge_sorted<KR>(top.v, lane);
+        bool twice[KR], any = false;
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            const uint64_t up = __shfl_up_sync(0xffffffffu, top.v[r], 1);
+            const uint64_t before = __shfl_sync(0xffffffffu, top.v[r > 0 ? r - 1 : 0], 31);
+            const uint64_t prev = lane ? up : (r > 0 ? before : kEmpty);
+            twice[r] = top.v[r] == prev && top.v[r] != kEmpty;
+            any |= twice[r];
+        }
+        if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+            for (int r = 0; r < KR; ++r)
+                if (twice[r]) top.v[r] = kEmpty;
+            sort_all<KR>(top.v, lane);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < KR; ++r) mine[r * 32 + lane] = top.v[r];
+    __syncwarp();
+}
+
 }  // namespace hc

@@ -1,5 +1,5 @@
 // Arguments and shared-memory layout of the walk kernels: one query per warp
-// (query.cu).
+// (query.cu), a query per several warps (query_split.cu).
 #pragma once
 
 #include "hc_dispatch.cuh"
@@ -10,6 +10,7 @@
 namespace hc {
 
 constexpr int kQWarps = 8;       // warps per block, a query each
+constexpr int kSplitWarps = 16;  // warps per block that share queries
 
 struct QueryArgs {
     IndexView ix;
@@ -29,5 +30,8 @@ template <int LPR>
 __host__ __device__ __forceinline__ uint32_t ring_bytes(uint32_t row_bytes) {
     return LPR <= 8 ? kRingRows * row_bytes : kWideRing;
 }
+
+// wpq (a power of two up to kSplitWarps) warps per query; no order
+cudaError_t launch_split(const QueryArgs& a, uint32_t wpq, cudaStream_t s);
 
 }  // namespace hc

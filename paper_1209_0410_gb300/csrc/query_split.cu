@@ -1,0 +1,92 @@
+// Small batches in arrival order: several warps to a query, so that a handful of
+// queries occupies the chip and a single one does not wait on a serial walk.
+// Bound by latency: the launch, two rounds of dependent loads for the key, four
+// or five for the search, then 1/16 of the steps (100,000 rows, p = 128: one query
+// 21 us against 56 with one warp; 1,000 queries at p = 64: 36 against 46 us).
+#include "hc_walk.cuh"
+
+namespace hc {
+
+namespace {
+
+// A small batch: wpq warps (a power of two up to kSplitWarps) share a query.
+// They search its lists with their lanes spread over the probes, walk every
+// wpq-th step each and merge their lists pairwise.
+template <bool F32, int LPR, int KR>
+__global__ void __launch_bounds__(kSplitWarps * 32, 1) split_kernel(QueryArgs a, uint32_t wpq) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t group = warp / wpq, sub = warp % wpq;
+    const uint32_t qi = blockIdx.x * (kSplitWarps / wpq) + group;
+    const bool mine = qi < a.nq;   // the others only take part in the barriers
+    const IndexView& ix = a.ix;
+    const uint8_t* qrow = static_cast<const uint8_t*>(a.q) + (size_t)(mine ? qi : 0) * ix.row_bytes;
+    const uint32_t rb = ring_bytes<LPR>(ix.row_bytes);
+    uint64_t* lists = reinterpret_cast<uint64_t*>(smem + kSplitWarps * rb);
+    uint64_t* list = lists + (size_t)warp * 32 * KR;
+    uint32_t* totals = reinterpret_cast<uint32_t*>(lists + kSplitWarps * 32 * KR);
+    uint32_t* pos_w = totals + kSplitWarps + group * 2 * ix.lists;
+    uint32_t* win_pre = pos_w + ix.lists;
+    if (mine) {
+        if (a.pos_in)
+            load_positions(ix, qrow, pos_w, lane, sub, wpq, a.pos_in + (size_t)qi * ix.lists,
+                           nullptr);
+        else
+            query_positions_spread(ix, qrow, pos_w, lane, sub, wpq);
+    }
+    __syncthreads();
+    if (mine && sub == 0) {
+        const uint32_t depth = a.p_query ? __ldg(a.p_query + qi) : a.p;
+        const uint32_t total = pack_windows(ix, depth, 0, 1, pos_w, pos_w, win_pre, lane);
+        if (lane == 0) totals[group] = total;
+    }
+    __syncthreads();
+    WarpTopK<KR> top;
+    top.init();
+    if (mine)
+        walk_packed<F32, LPR, KR, true, true>(ix, qrow, a.k, pos_w, win_pre, ix.lists,
+                                              totals[group], sub, wpq, smem + warp * rb, top,
+                                              lane);
+#pragma unroll
+    for (int r = 0; r < KR; ++r) list[r * 32 + lane] = top.v[r];
+    for (uint32_t step = 1; step < wpq; step *= 2) {
+        __syncthreads();
+        if (sub % (2 * step) == 0)
+            merge_lists<KR>(list, list + (size_t)step * 32 * KR, a.k, lane);
+    }
+    if (mine && sub == 0) {
+#pragma unroll
+        for (int r = 0; r < KR; ++r) top.v[r] = list[r * 32 + lane];
+        top.template store<F32>(a.k, lane, a.out_ids + (size_t)qi * a.k,
+                                static_cast<uint32_t*>(a.out_dist) + (size_t)qi * a.k);
+    }
+}
+
+template <bool F32, int LPR, int KR>
+struct SplitLaunch {
+    static cudaError_t run(const QueryArgs& a, uint32_t wpq, cudaStream_t s) {
+        if constexpr (KR == 2) {
+            return cudaErrorInvalidValue;   // launch_split takes 4
+        } else {
+            const uint32_t per = kSplitWarps / wpq;   // queries per block
+            const size_t smem = kSplitWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 256 * KR + 4) +
+                                8ull * per * a.ix.lists;
+            const cudaError_t e =
+                cudaFuncSetAttribute(split_kernel<F32, LPR, KR>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            split_kernel<F32, LPR, KR><<<(a.nq + per - 1) / per, kSplitWarps * 32, smem, s>>>(a, wpq);
+            count_launches(1);
+            return cudaGetLastError();
+        }
+    }
+};
+
+}  // namespace
+
+cudaError_t launch_split(const QueryArgs& a, uint32_t wpq, cudaStream_t s) {
+    return dispatch<SplitLaunch>(a.ix.P.dtype == HC_F32, lanes_per_row(a.ix.row_bytes),
+                                 a.k <= 32 ? 1 : 4, a, wpq, s);
+}
+
+}  // namespace hc
