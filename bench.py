@@ -45,6 +45,7 @@ DATA = ("synthetic: seeded 64-cluster isotropic Gaussian mixture (centres unifor
         "database rows plus N(0, 8) noise")
 QUERY_SOURCES = ["paper_1209_0410_gb300/csrc/query.cu", "paper_1209_0410_gb300/csrc/hc_topk.cuh",
                  "paper_1209_0410_gb300/csrc/hc_walk.cuh",
+                 "paper_1209_0410_gb300/csrc/query_sweep.cu",
                  "paper_1209_0410_gb300/csrc/hc_device.cuh",
                  "paper_1209_0410_gb300/csrc/hc_query_dev.cuh"]
 

@@ -904,4 +904,68 @@ __device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t*
                                             top, lane);
 }
 
+// The walk of a query's packed windows in the order of the row ids, kSweep
+// entries at a time (a sweep): the ids of a sweep are sorted into 256 buckets of
+// row ranges (a counting sort in shared memory) before its rows are read.  The
+// warps of a block start every sweep together, so that at any time the SM reads
+// rows of a small part of the database, whatever order the lists hold them in.
+// counts: 256 words, sorted: kSweep words per warp.  Every warp of the block
+// calls this, with total = 0 when it has no query.
+constexpr int kSweepLoads = 32;
+constexpr uint32_t kSweep = 32 * kSweepLoads;
+
+template <bool F32, int LPR, int KR, bool FULL>
+__device__ __forceinline__ void walk_sweeps(const IndexView& ix, const uint8_t* qrow, uint32_t k,
+                                            const uint32_t* win_at, const uint32_t* win_pre,
+                                            uint32_t nm, uint32_t total, uint32_t shift,
+                                            uint32_t* counts, uint32_t* sorted, uint8_t* ring,
+                                            WarpTopK<KR>& top, int lane) {
+    StagedSteps<F32, LPR, KR, FULL, true> pipe(ix, qrow, ring, top, k);
+    WindowCursor cur;
+    const uint32_t sweeps = total / kSweep + (total % kSweep != 0);
+    for (uint32_t s = 0; __syncthreads_or(s < sweeps); ++s) {
+        if (s >= sweeps) continue;
+        const uint32_t e0 = s * kSweep, cnt = min(kSweep, total - e0);
+        uint32_t id[kSweepLoads];
+#pragma unroll
+        for (int u = 0; u < kSweepLoads; ++u)
+            id[u] = cur.id(ix, win_at, win_pre, nm, total,
+                           e0 + min(32 * (uint32_t)u + (uint32_t)lane, cnt - 1));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) counts[32 * j + lane] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kSweepLoads; ++u)
+            if (32 * (uint32_t)u + (uint32_t)lane < cnt) atomicAdd(&counts[id[u] >> shift], 1u);
+        __syncwarp();
+        // exclusive prefixes: lane l owns buckets 8 l .. 8 l + 7
+        uint4 lo4 = reinterpret_cast<const uint4*>(counts)[2 * lane];
+        uint4 hi4 = reinterpret_cast<const uint4*>(counts)[2 * lane + 1];
+        const uint32_t sum = lo4.x + lo4.y + lo4.z + lo4.w + hi4.x + hi4.y + hi4.z + hi4.w;
+        uint32_t run = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += y;
+        }
+        run -= sum;
+        uint4 a, b;
+        a.x = run, a.y = a.x + lo4.x, a.z = a.y + lo4.y, a.w = a.z + lo4.z;
+        b.x = a.w + lo4.w, b.y = b.x + hi4.x, b.z = b.y + hi4.y, b.w = b.z + hi4.z;
+        reinterpret_cast<uint4*>(counts)[2 * lane] = a;
+        reinterpret_cast<uint4*>(counts)[2 * lane + 1] = b;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kSweepLoads; ++u)
+            if (32 * (uint32_t)u + (uint32_t)lane < cnt)
+                sorted[atomicAdd(&counts[id[u] >> shift], 1u)] = id[u];
+        __syncwarp();
+        for (uint32_t o = 0; o < cnt; o += 32) {
+            const uint32_t n = min(32u, cnt - o);
+            pipe.add(sorted[o + min((uint32_t)lane, n - 1)], n, top, k, lane);
+        }
+    }
+    pipe.finish(top, k, lane);
+}
+
 }  // namespace hc

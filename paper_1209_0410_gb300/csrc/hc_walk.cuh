@@ -1,5 +1,6 @@
 // Arguments and shared-memory layout of the walk kernels: one query per warp
-// (query.cu), a query per several warps (query_split.cu).
+// (query.cu), a query per several warps (query_split.cu), rows in sweeps of
+// ascending ids (query_sweep.cu).
 #pragma once
 
 #include "hc_dispatch.cuh"
@@ -31,6 +32,8 @@ __host__ __device__ __forceinline__ uint32_t ring_bytes(uint32_t row_bytes) {
     return LPR <= 8 ? kRingRows * row_bytes : kWideRing;
 }
 
+// uint8 rows of at most 128 bytes; order and pos_cm set
+cudaError_t launch_sweeps(const QueryArgs& a, cudaStream_t s);
 // wpq (a power of two up to kSplitWarps) warps per query; no order
 cudaError_t launch_split(const QueryArgs& a, uint32_t wpq, cudaStream_t s);
 

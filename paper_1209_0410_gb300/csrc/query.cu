@@ -238,6 +238,9 @@ __global__ void __launch_bounds__(256) fence_kernel(const uint64_t* __restrict__
         fence[j] = __ldg(keys_hi + (j << kFenceShift)) & kFenceMask;
 }
 
+// How a batch is walked (walk_kind).
+enum Walk { kPlain, kByPartition, kSweeps };
+
 template <bool F32, int LPR, int KR>
 struct QueryLaunch {
     template <typename K>
@@ -250,12 +253,39 @@ struct QueryLaunch {
         count_launches(1);
         return cudaGetLastError();
     }
-    static cudaError_t run(const QueryArgs& a, cudaStream_t s) {
+    static cudaError_t run(const QueryArgs& a, bool by_partition, cudaStream_t s) {
         const size_t smem =
             kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 2 * sizeof(uint32_t) * a.ix.lists);
+        if constexpr (LPR <= 8 && !F32)
+            if (by_partition) return go(query_kernel<F32, LPR, KR, 2>, a, smem, s);
         return go(query_kernel<F32, LPR, KR, 3>, a, smem, s);
     }
 };
+
+// The address translation of an SM reaches 256 MB (128 pages of 2 MB: random
+// 128-byte rows of up to 256 MB arrive at 22 TB/s, of 384 MB at 8.4, of 1.2 GB at
+// 5.7, all of them in L2).  A batch in key order reads its rows of a larger
+// database
+//   kByPartition  when a partition's rows are within reach: the walk goes
+//                 partition by partition as it is, and with 16 instead of 24
+//                 warps per SM they stay in the same one (8 partitions of 160
+//                 MB, 100,000 queries at p = 32: 4.2 against 6.3 ms, sweeps 4.6);
+//   kSweeps       otherwise, sorted by row id (100,000 queries at p = 128 on 10M
+//                 rows: 2.5 against 3.9 ms; 20M 3.0 against 4.2, 50M 3.8 against
+//                 4.4; 3M rows, 384 MB: 2.4 against 2.7; 1.5M rows, 192 MB: 2.4
+//                 against 1.8, so the line lies between).
+// In arrival order the rows come from DRAM, which then binds (sweeps 4.6 against
+// 4.2 ms), and rows wider than 128 bytes need fewer translations per byte.
+constexpr uint64_t kReachBytes = 320ull << 20;
+
+Walk walk_kind(const QueryArgs& a) {
+    const IndexView& ix = a.ix;
+    const uint64_t bytes = ix.rows * ix.row_bytes, parts = ix.lists / ix.P.curves;
+    if (!a.pos_cm || ix.P.dtype != HC_U8 || ix.row_bytes > 128 || bytes < kReachBytes)
+        return kPlain;
+    if (parts > 1 && bytes / parts < (200ull << 20)) return kByPartition;
+    return ix.lists <= 96 ? kSweeps : kPlain;   // two blocks' shared memory per SM
+}
 
 // Warps per query when a batch in arrival order would leave SMs idle: as many as
 // one block of kSplitWarps warps per SM still holds (a second block waits for
@@ -282,8 +312,10 @@ cudaError_t launch_query(const IndexView& ix, const void* q, uint32_t nq, uint32
     QueryArgs a{ix, q, nq, k, p, out_ids, out_dist, nullptr, p_query, pos_in, order, pos_cm};
     const uint32_t wpq = split_warps(a);
     if (wpq > 1) return launch_split(a, wpq, s);
+    const Walk walk = walk_kind(a);
+    if (walk == kSweeps) return launch_sweeps(a, s);
     return dispatch<QueryLaunch>(ix.P.dtype == HC_F32, lanes_per_row(ix.row_bytes), regs_for_k(k),
-                                 a, s);
+                                 a, walk == kByPartition, s);
 }
 
 cudaError_t launch_order_keys(const IndexView& ix, const void* q, uint32_t nq, uint32_t ncurves,

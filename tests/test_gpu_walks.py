@@ -1,5 +1,6 @@
 """The walks a batch may take -- a warp per query, several warps per query (small
-batches) -- give the same ids and the same distance bits: every row's
+batches), a database in sweeps of ascending ids or partition by partition (large
+databases, key order) -- give the same ids and the same distance bits: every row's
 distance is summed in one order whoever reads it.  (The warp-per-query walk and the
 small batches are checked against the oracle in test_gpu_parity.py and
 test_gpu_scale.py.)"""
@@ -60,3 +61,19 @@ def test_small_batches_equal_large(n, d, dtype, curves, m, parts, k, p, few):
         assert same(hc.hc_query_at(idx, qs, k, p, pos), [t[s] for t in want]), b
         at += b
     assert same(hc.hc_query_ordered(idx, q, k, p), want)
+
+
+@pytest.mark.parametrize("d,curves,m,parts,k,p,nq", [
+    (128, 8, 16, 1, 10, 64, 203), (128, 8, 16, 1, 10, 65, 8), (128, 8, 16, 1, 33, 192, 3000),
+    (128, 8, 16, 1, 128, 7, 65), (128, 3, 16, 1, 1, 1, 7), (64, 4, 16, 1, 10, 128, 203),
+    (64, 4, 8, 1, 10, 129, 203), (16, 1, 16, 1, 10, 512, 99), (48, 3, 16, 1, 40, 171, 99),
+    (112, 7, 16, 1, 10, 300, 99), (128, 8, 16, 2, 10, 40, 203), (64, 4, 16, 2, 100, 17, 203),
+    (128, 8, 16, 12, 10, 9, 203), (128, 8, 16, 13, 10, 9, 203)])
+def test_large_databases_in_key_order(d, curves, m, parts, k, p, nq):
+    """350 MB of rows, above the reach of an SM's address translation: sweeps, whole
+    and cut ones, and the walk partition by partition."""
+    from paper_1209_0410_gb300 import hc
+    db, q = make((350 << 20) // d + 13, d, "u8", nq, d + p)
+    idx = hc.hc_build(db, curves, m, partitions=parts)
+    assert same(hc.hc_query_ordered(idx, q, k, p), hc.hc_query(idx, q, k, p))
+    assert same(hc.hc_query_ordered(idx, q, k, 0), hc.hc_query(idx, q, k, 0))
