@@ -9,9 +9,10 @@
 // constants -32768 (on twice the digit), -256 and -1.
 //
 // One block (one per SM) holds MT x 128 queries as the A operand and streams a
-// share of the rows as B tiles of NB; the shares of one query tile are the
-// blocks of a cluster, whose per-query lists meet in distributed shared memory
-// at the end, so nothing is allocated.  Warps:
+// share of the rows as B tiles of NB.  At the end the per-query lists of a
+// cluster's blocks meet in distributed shared memory, and each cluster merges its
+// lists into the output rows under a lock per row (the row's first id word), so
+// nothing is allocated and every SM has a share.  Warps:
 //   0 .. 4 MT - 1   epilogue, one query per thread (tensor-memory lane): the
 //                   scores against the query's threshold; the few that pass are
 //                   appended to the query's list in shared memory, which the
@@ -24,15 +25,16 @@
 // per stage.
 //
 // Bound: the tensor cores' dense float16 rate (5.1 TFLOP for 2,000 queries on
-// 10M rows of 128, 2.6 ms at 1940 TFLOP/s over 152 SMs).  Measured there: 7.1
-// ms against 633 ms with vabsdiff and dp4a, one warp per query; 6.35 ms without
-// a candidate ever passing.  Clusters of 12 leave 56 SMs idle (96 run), and a
-// stage waits for its refill (one query tile per block, half the tensor work,
-// takes 1,260 cycles per row tile where two take 1,850).
+// 10M rows of 128, 2.6 ms at 1940 TFLOP/s).  Measured there: 5.0 ms against 633 ms
+// with vabsdiff and dp4a, one warp per query (7.1 with one cluster of 12 blocks
+// per query tile, which left 56 SMs idle); one query: 0.63 ms.  A stage waits for
+// its refill: one query tile per block, half the tensor work, takes 1,260 cycles
+// per row tile where two take 1,850.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "hc_internal.h"
 #include "hc_query_dev.cuh"
@@ -69,9 +71,20 @@ struct BruteArgs {
     const uint8_t* q;
     uint64_t n;
     uint32_t row_bytes, nq, k;
+    uint32_t groups;   // clusters that share a query tile
     int32_t* out_ids;
     uint32_t* out_dist;
 };
+
+constexpr int32_t kLocked = -3;   // no id: ids are >= 0, -1 marks an empty slot
+
+// empty output rows, which the clusters then merge into
+__global__ void __launch_bounds__(256) empty_rows_kernel(uint64_t n, int32_t* ids, uint32_t* dist) {
+    const uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    ids[i] = -1;
+    dist[i] = 0x7FFFFFFFu;
+}
 
 // 16 uint8 coordinates, shifted by -128, as float16 (bytes 0x64 above each
 // coordinate make 1024 + x; 1152 is subtracted)
@@ -164,7 +177,8 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     const uint32_t bar_drained = bar_done + 8 * kBBufs;        // accumulators read
 
     cg::cluster_group cluster = cg::this_cluster();
-    const uint32_t share = cluster.block_rank(), shares = cluster.num_blocks();
+    const uint32_t rank = cluster.block_rank(), blocks = cluster.num_blocks();
+    const uint32_t shares = blocks * a.groups, share = blockIdx.x % shares;
     const uint32_t q0 = (blockIdx.x / shares) * S::kQueries;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t tiles = (a.n + NB - 1) / NB;
@@ -405,57 +419,92 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
         tc_fence_after();
         tmem_free(tmem, S::kCols);
     }
-    // Queries are dealt out to the cluster's blocks: each merges every share's
-    // sorted list of its queries (the smaller of entry e of one and entry
-    // KS - 1 - e of the other are the KS smallest, a bitonic sequence) and
-    // writes the result.
+    // Queries are dealt out to the cluster's blocks: each merges every block's
+    // sorted list of its queries (the smaller of entry e of one and entry KS - 1 -
+    // e of the other are the KS smallest, a bitonic sequence) and puts the result
+    // out.  The clusters of a tile begin at different queries.
     cluster.sync();
     constexpr int KR = KS / 32, kWarps = S::kThreads / 32;
-    for (uint32_t ql = share + shares * (uint32_t)warp; ql < (uint32_t)S::kQueries;
-         ql += shares * kWarps) {
-        if (q0 + ql >= a.nq) break;
+    const uint32_t turn = S::kQueries / blocks / kWarps * (share / blocks) / a.groups;
+    const uint32_t rounds = (S::kQueries + blocks * kWarps - 1) / (blocks * kWarps);
+    for (uint32_t i = 0; i < rounds; ++i) {
+        const uint32_t ql = rank + blocks * ((uint32_t)warp + kWarps * ((i + turn) % rounds));
+        if (ql >= (uint32_t)S::kQueries || q0 + ql >= a.nq) continue;
+        int32_t* ids = a.out_ids + (size_t)(q0 + ql) * a.k;
+        uint32_t* dist = a.out_dist + (size_t)(q0 + ql) * a.k;
         WarpTopK<KR> top;
         top.init();
-        for (uint32_t b = 0; b < shares; ++b) {
+        for (uint32_t b = 0; b < blocks; ++b) {
             const uint64_t* other = cluster.map_shared_rank(lists + (size_t)ql * KS, b);
 #pragma unroll
             for (int r = 0; r < KR; ++r)
                 top.v[r] = min(top.v[r], other[KS - 1 - (r * 32 + lane)]);
             merge_sorted<KR>(top.v, lane);
         }
-        top.template store<false>(a.k, lane, a.out_ids + (size_t)(q0 + ql) * a.k,
-                                  a.out_dist + (size_t)(q0 + ql) * a.k);
+        if (a.groups == 1) {
+            top.template store<false>(a.k, lane, ids, dist);
+            continue;
+        }
+        // take the row: its first id word says kLocked meanwhile
+        int32_t first = kLocked;
+        if (lane == 0) {
+            const uint64_t t = global_ns();
+            do first = atomicExch(ids, kLocked);
+            while (first == kLocked && global_ns() - t < kMbarLimitNs);
+        }
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (first == kLocked) continue;   // never: a holder lets go in microseconds
+        __threadfence();
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            const uint32_t e = KS - 1 - (r * 32 + lane);   // reversed, as above
+            const int32_t id = e >= a.k ? -1 : (e == 0 ? first : __ldcg(ids + e));
+            const uint64_t x =
+                id < 0 ? kEmpty : ((uint64_t)__ldcg(dist + e) << 32) | (uint32_t)id;
+            top.v[r] = min(top.v[r], x);
+        }
+        merge_sorted<KR>(top.v, lane);
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+            const uint32_t e = r * 32 + lane;
+            if (e >= a.k) continue;
+            const bool empty = top.v[r] == kEmpty;
+            if (e > 0) __stcg(ids + e, empty ? -1 : (int32_t)(uint32_t)top.v[r]);
+            __stcg(dist + e, empty ? 0x7FFFFFFFu : (uint32_t)(top.v[r] >> 32));
+        }
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicExch(ids, top.v[0] == kEmpty ? -1 : (int32_t)(uint32_t)top.v[0]);
     }
     cluster.sync();
 }
 
-// Shares (blocks of a cluster) per query tile: the cluster size that finishes
-// `qtiles` tiles soonest, where fit[c] clusters of c blocks run at once (a
-// cluster lies within one GPC, whose SMs need not be a multiple of its size).
-// Every share has at least two row tiles to stream.
-uint32_t pick_shares(const int (&fit)[17], uint64_t qtiles, uint64_t btiles) {
-    uint32_t best = 1;
-    double best_time = 1e300;
-    for (uint32_t c = 1; c <= 16; ++c) {
-        if (c > 1 && btiles < 2 * c) break;
-        if (fit[c] < 1) continue;
-        const double time = (double)((qtiles + fit[c] - 1) / fit[c]) / c;
-        if (time < best_time) {
-            best_time = time;
-            best = c;
-        }
+// How a query tile's rows are shared out: `blocks` per cluster (their lists meet
+// in shared memory), `groups` clusters per tile (each merges its lists into the
+// output rows, one after the other when they end together: about 3.5 us each).
+// A row tile takes a block about 0.65 us, so more than sqrt(btiles / 10.8)
+// clusters of two cost more than they save; up to that the chip is filled (`fit`
+// clusters of two at once).  A few row tiles are left to one cluster of eight.
+struct Sharing {
+    uint32_t blocks, groups;
+};
+Sharing pick_sharing(uint32_t fit, uint64_t qtiles, uint64_t btiles) {
+    if (btiles < 256) {
+        uint32_t blocks = 8;
+        while (blocks > 1 && btiles < 2 * blocks) blocks /= 2;
+        return {blocks, 1};
     }
-    return best;
+    const uint64_t chip = std::max<uint64_t>(1, fit / qtiles);
+    const uint64_t worth = (uint64_t)std::sqrt((double)btiles / 10.8);
+    return {2, (uint32_t)std::min(chip, worth)};
 }
 
 template <int ATOMS, int KS, int MT>
-cudaError_t launch_tensor(const BruteArgs& a, cudaStream_t s) {
+cudaError_t launch_tensor(BruteArgs a, cudaStream_t s) {
     using S = BruteShape<ATOMS, KS, MT>;
     auto kernel = brute_tensor_kernel<ATOMS, KS, MT>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)S::kSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
@@ -466,19 +515,22 @@ cudaError_t launch_tensor(const BruteArgs& a, cudaStream_t s) {
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    int fit[17] = {0};
-    for (uint32_t c = 1; c <= 16; ++c) {
-        at.val.clusterDim.x = c;
-        cfg.gridDim = dim3(c);
-        if (cudaOccupancyMaxActiveClusters(&fit[c], kernel, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            fit[c] = 0;
-        }
-    }
+    at.val.clusterDim.x = 2;
+    cfg.gridDim = dim3(2);
+    int fit = 0;
+    if ((e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg)) != cudaSuccess) return e;
     const uint64_t qtiles = ((uint64_t)a.nq + S::kQueries - 1) / S::kQueries;
-    const uint32_t shares = pick_shares(fit, qtiles, (a.n + S::NB - 1) / S::NB);
-    at.val.clusterDim.x = shares;
-    cfg.gridDim = dim3((unsigned)(qtiles * shares));
+    const Sharing sharing =
+        pick_sharing((uint32_t)std::max(fit, 1), qtiles, (a.n + S::NB - 1) / S::NB);
+    a.groups = sharing.groups;
+    at.val.clusterDim.x = sharing.blocks;
+    cfg.gridDim = dim3((unsigned)(qtiles * a.groups * sharing.blocks));
+    if (a.groups > 1) {
+        const uint64_t slots = (uint64_t)a.nq * a.k;
+        empty_rows_kernel<<<(unsigned)((slots + 255) / 256), 256, 0, s>>>(slots, a.out_ids,
+                                                                         a.out_dist);
+        count_launches(1);
+    }
     e = cudaLaunchKernelEx(&cfg, kernel, a);
     count_launches(1);
     return e == cudaSuccess ? cudaGetLastError() : e;
@@ -497,10 +549,9 @@ cudaError_t launch_brute_tensor(const void* db, uint64_t n, uint32_t row_bytes, 
                                 uint32_t nq, uint32_t k, int32_t* out_ids, void* out_dist,
                                 cudaStream_t s) {
     const BruteArgs a{static_cast<const uint8_t*>(db), static_cast<const uint8_t*>(q), n,
-                      row_bytes, nq, k, out_ids, static_cast<uint32_t*>(out_dist)};
-    // two query tiles per block (half the row conversions) once single tiles
-    // in clusters of 16 would not all run at once
-    const bool two = nq > 128 * 7;
+                      row_bytes, nq, k, 1, out_ids, static_cast<uint32_t*>(out_dist)};
+    // two query tiles per block halve the row conversions
+    const bool two = nq > 128;
     if (row_bytes <= 64) {
         if (k > 16) return launch_tensor<1, 128, 1>(a, s);
         return two ? launch_tensor<1, 32, 2>(a, s) : launch_tensor<1, 32, 1>(a, s);
