@@ -13,9 +13,10 @@
 //   training   two FP32 kernels per step: the layers forward and back for 32
 //              samples per block, then every weight's gradient and Adam update
 //   inference  BF16 inputs and weights, FP32 accumulation, fused with the
-//              feature computation: one warp per query
+//              feature computation: one, two or four queries per warp
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -529,36 +530,79 @@ struct MlpView {
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-// y of one sample whose raw features sit in xs[0..in) (warp-shared memory).
+// y of G samples whose raw features sit in xs[i * G + g] (warp-shared memory).
 // Weights in shared memory (bf16), inputs of each layer rounded to bf16,
-// accumulation in float32.  Lane j computes hidden units j and j + 32.
-__device__ float mlp_warp_forward(const MlpView& V, const __nv_bfloat16* sW1,
-                                  const __nv_bfloat16* sW2, const __nv_bfloat16* sW3,
-                                  const float* sb, float* xs, float* hs, int lane) {
+// accumulation in float32, inputs ascending.  Lane j computes hidden units j and
+// j + 32 of all G samples: a weight is read and widened once for them, and an
+// input of all of them is one load (G = 4: 13 instructions for 8 FMAs; one
+// sample and one unit at a time took 4 for each).
+template <int G>
+__device__ __forceinline__ void mlp_layer(const __nv_bfloat16* w, uint32_t in, uint32_t out,
+                                          const float* xs, int lane, float (&acc)[2][G]) {
+    const __nv_bfloat16* w0 = w + min((uint32_t)lane, out - 1);
+    const __nv_bfloat16* w1 = w + min((uint32_t)lane + 32, out - 1);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int g = 0; g < G; ++g) acc[u][g] = 0.f;
+#pragma unroll 4
+    for (uint32_t i = 0; i < in; ++i) {
+        const float v0 = __bfloat162float(w0[i * out]), v1 = __bfloat162float(w1[i * out]);
+        float x[G];
+        if constexpr (G == 4)
+            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xs + 4 * i);
+        else
+#pragma unroll
+            for (int g = 0; g < G; ++g) x[g] = xs[i * G + g];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            acc[0][g] = fmaf(x[g], v0, acc[0][g]);
+            acc[1][g] = fmaf(x[g], v1, acc[1][g]);
+        }
+    }
+}
+
+template <int G>
+__device__ void mlp_warp_forward(const MlpView& V, const __nv_bfloat16* sW1,
+                                 const __nv_bfloat16* sW2, const __nv_bfloat16* sW3,
+                                 const float* sb, float* xs, float* hs, int lane, float (&y)[G]) {
     const float* b1 = sb;
     const float* b2 = sb + kMaxDim;
     const float b3 = sb[2 * kMaxDim];
     const float* mu = sb + 2 * kMaxDim + 1;
     const float* isd = mu + kMaxDim;
-    for (uint32_t i = lane; i < V.in; i += 32) xs[i] = bf((xs[i] - mu[i]) * isd[i]);
+    for (uint32_t i = lane; i < V.in; i += 32)
+#pragma unroll
+        for (int g = 0; g < G; ++g) xs[i * G + g] = bf((xs[i * G + g] - mu[i]) * isd[i]);
     __syncwarp();
-    for (uint32_t j = lane; j < V.h1; j += 32) {
-        float a = 0.f;
-        for (uint32_t i = 0; i < V.in; ++i) a = fmaf(xs[i], __bfloat162float(sW1[i * V.h1 + j]), a);
-        hs[j] = bf(fmaxf(a + b1[j], 0.f));
+    float acc[2][G];
+    mlp_layer<G>(sW1, V.in, V.h1, xs, lane, acc);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const uint32_t j = (uint32_t)lane + 32 * u;
+        if (j < V.h1)
+#pragma unroll
+            for (int g = 0; g < G; ++g) hs[j * G + g] = bf(fmaxf(acc[u][g] + b1[j], 0.f));
     }
     __syncwarp();
-    float part = 0.f;
-    for (uint32_t j = lane; j < V.h2; j += 32) {
-        float a = 0.f;
-        for (uint32_t i = 0; i < V.h1; ++i) a = fmaf(hs[i], __bfloat162float(sW2[i * V.h2 + j]), a);
-        const float h2v = bf(fmaxf(a + b2[j], 0.f));
-        part = fmaf(h2v, __bfloat162float(sW3[j]), part);
+    mlp_layer<G>(sW2, V.h1, V.h2, hs, lane, acc);
+#pragma unroll
+    for (int g = 0; g < G; ++g) y[g] = 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const uint32_t j = (uint32_t)lane + 32 * u;
+        if (j < V.h2)
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                y[g] = fmaf(bf(fmaxf(acc[u][g] + b2[j], 0.f)), __bfloat162float(sW3[j]), y[g]);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    for (int g = 0; g < G; ++g) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) y[g] += __shfl_xor_sync(0xffffffffu, y[g], o);
+        y[g] += b3;
+    }
     __syncwarp();
-    return part + b3;
 }
 
 // Stages bf16 weights and float biases / normalisation in shared memory.
@@ -597,17 +641,18 @@ __global__ void __launch_bounds__(kPredWarps * 32) mlp_infer_kernel(MlpView V,
     for (uint32_t i = blockIdx.x * kPredWarps + warp; i < n; i += gridDim.x * kPredWarps) {
         for (uint32_t j = lane; j < V.in; j += 32) xs[j] = x[(size_t)i * V.in + j];
         __syncwarp();
-        const float yi = mlp_warp_forward(V, sW, sW + V.in * V.h1, sW + V.in * V.h1 + V.h1 * V.h2,
-                                          sb, xs, hs, lane);
-        if (lane == 0) y[i] = yi;
+        float yi[1];
+        mlp_warp_forward<1>(V, sW, sW + V.in * V.h1, sW + V.in * V.h1 + V.h1 * V.h2, sb, xs, hs,
+                            lane, yi);
+        if (lane == 0) y[i] = yi[0];
         __syncwarp();
     }
 }
 
-size_t pred_smem(const MlpView& V) {
+size_t pred_smem(const MlpView& V, int G = 1) {
     const uint32_t nw = V.in * V.h1 + V.h1 * V.h2 + V.h2;
     return ((nw * 2 + 15) & ~15u) + sizeof(float) * (4 * kMaxDim + 1 + 3) +
-           sizeof(float) * kPredWarps * 2 * kMaxDim + sizeof(uint32_t) * kPredWarps * (64 + 128);
+           sizeof(float) * kPredWarps * 2 * kMaxDim * G + sizeof(uint32_t) * kPredWarps * (64 + 128);
 }
 
 // ------------------------------------------------------------ features
@@ -630,17 +675,39 @@ __device__ __forceinline__ float key_gap_octave(uint64_t ah, uint64_t al, uint64
     return octave128(gh, gl);
 }
 
-// The 4 * curves features of one query into xs (warp-shared), from the
-// positions pos_w of lists 0..curves-1 (khi/klo: lane c holds curve c's key).
+// Whether the low words of two keys whose high words differ by dh cannot show in
+// the octave of their gap: its top bit and the 16 below lie in dh, above bits of
+// dh that are not all zero, so a borrow from the low words ends below them.  Holds
+// for all but one gap in thousands of a long list, whose low word (the row's key
+// where the index keeps high words only) is then not computed.
+__device__ __forceinline__ bool gap_from_high(uint64_t dh) {
+    const int e = 63 - __clzll((long long)dh);
+    return e > 16 && (dh & ((1ull << (e - 16)) - 1));
+}
+
+// The 4 * curves features of one query into xs (warp-shared, feature i at
+// xs[i * stride]), from the positions pos_w of lists 0..curves-1 (khi/klo: lane c holds curve c's key).
 // All curves at once: the 8-entry centre windows fill 32-row steps (slot
 // 8 c + j = entry j of curve c's window, distances parked in sd), and lanes
 // 2 c, 2 c + 1 take curve c's predecessor and successor gaps (a low key word
 // recomputed from its row where the index keeps high words only).
 __device__ void query_features(const IndexView& ix, const uint8_t* qrow, uint4 qv0,
                                const uint32_t* pos_w, uint64_t khi, uint64_t klo, float* xs,
-                               uint32_t* sd, int lane) {
+                               uint32_t* sd, int lane, uint32_t stride = 1) {
     const uint8_t* db = static_cast<const uint8_t*>(ix.db);
     const uint32_t C = ix.P.curves;
+    // the loads of the gaps first: lanes 2c, 2c + 1 the predecessor and the
+    // successor of curve c's key
+    const uint32_t gc = (uint32_t)lane / 2 < C ? (uint32_t)lane / 2 : 0u;
+    bool near = (uint32_t)lane / 2 < C;
+    uint64_t ge = 0, gh = 0;
+    {
+        const uint64_t off = ix.list_off[gc];
+        const uint32_t n = (uint32_t)(ix.list_off[gc + 1] - off), pos = pos_w[gc];
+        near = near && ((lane & 1) ? pos < n : pos > 0);
+        ge = off + pos - ((lane & 1) ? 0 : 1);
+        if (near) gh = ix.keys_hi[ge];
+    }
     // centre window of curve c = lane / 8 (per slot)
     for (uint32_t t = 0; t < C; t += 4) {
         const uint32_t c = t + (uint32_t)lane / 8, j = (uint32_t)lane % 8;
@@ -665,21 +732,16 @@ __device__ void query_features(const IndexView& ix, const uint8_t* qrow, uint4 q
     __syncwarp();
     float f0 = kFeatNone, f1 = kFeatNone, f2 = kFeatNone, f3 = kFeatNone;
     {
-        // lanes 2c, 2c+1: predecessor / successor gap of curve c
-        const uint32_t c = (uint32_t)lane / 2;
-        const uint64_t kh = __shfl_sync(0xffffffffu, khi, (int)(c < C ? c : 0));
-        const uint64_t kl = __shfl_sync(0xffffffffu, klo, (int)(c < C ? c : 0));
+        const uint64_t kh = __shfl_sync(0xffffffffu, khi, (int)gc);
+        const uint64_t kl = __shfl_sync(0xffffffffu, klo, (int)gc);
         float gap = kFeatNone;
-        if (c < C) {
-            const uint64_t off = ix.list_off[c];
-            const uint32_t n = (uint32_t)(ix.list_off[c + 1] - off);
-            const uint32_t pos = pos_w[c];
-            if ((lane & 1) == 0 && pos > 0) {
-                const uint64_t g = off + pos - 1;
-                gap = key_gap_octave(kh, kl, ix.keys_hi[g], entry_key_lo(ix, c, g));
-            } else if ((lane & 1) == 1 && pos < n) {
-                const uint64_t g = off + pos;
-                gap = key_gap_octave(ix.keys_hi[g], entry_key_lo(ix, c, g), kh, kl);
+        if (near) {
+            const uint64_t dh = (lane & 1) ? gh - kh : kh - gh;
+            if (gap_from_high(dh)) {
+                gap = octave128(dh, 0);
+            } else {
+                const uint64_t gl = entry_key_lo(ix, gc, ge);
+                gap = (lane & 1) ? key_gap_octave(gh, gl, kh, kl) : key_gap_octave(kh, kl, gh, gl);
             }
         }
         const float other = __shfl_xor_sync(0xffffffffu, gap, 1);
@@ -707,10 +769,10 @@ __device__ void query_features(const IndexView& ix, const uint8_t* qrow, uint4 q
     const float g0 = __shfl_sync(0xffffffffu, f0, (2 * lane) & 31);
     const float g1 = __shfl_sync(0xffffffffu, f1, (2 * lane) & 31);
     if ((uint32_t)lane < C) {
-        xs[4 * lane + 0] = g0;
-        xs[4 * lane + 1] = g1;
-        xs[4 * lane + 2] = f2;
-        xs[4 * lane + 3] = f3;
+        xs[(4 * lane + 0) * stride] = g0;
+        xs[(4 * lane + 1) * stride] = g1;
+        xs[(4 * lane + 2) * stride] = f2;
+        xs[(4 * lane + 3) * stride] = f3;
     }
     __syncwarp();
 }
@@ -747,7 +809,16 @@ __global__ void __launch_bounds__(kPredWarps * 32) features_kernel(IndexView ix,
         feat[(size_t)qi * 4 * ix.P.curves + j] = s_x[warp][j];
 }
 
-// features -> MLP -> p = clamp(ceil(2^(y + margin)), p_lo, p_hi), per query
+// features -> MLP -> p = clamp(ceil(2^(y + margin)), p_lo, p_hi), per query.
+// A warp takes G queries at once (at most 32 / G curves): lane g * 32 / G + c
+// computes curve c's key and position of query g, so that the keys and the
+// dependent loads of the searches, which fill `curves` lanes for one query, are
+// done for all of them together, and the layers read every weight once.  Bound by
+// the latency of scattered loads (long scoreboard half of the stalls, 45% of the
+// issue slots): of 590 us for 100,000 queries on 10M rows and 8 curves the searches
+// are 265, the keys 146, the 64 rows of each query's features 143, the layers 65;
+// one query per warp, every gap's low word computed: 1,025 us.
+template <int G>
 __global__ void __launch_bounds__(kPredWarps * 32, 4) predict_depths_kernel(
     IndexView ix, MlpView V, const uint8_t* q, uint32_t nq, float margin, uint32_t p_lo,
     uint32_t p_hi, uint32_t* p_out) {
@@ -756,30 +827,65 @@ __global__ void __launch_bounds__(kPredWarps * 32, 4) predict_depths_kernel(
     const uint32_t nw = V.in * V.h1 + V.h1 * V.h2 + V.h2;
     float* sb = reinterpret_cast<float*>(smem_raw + ((nw * 2 + 15) & ~15u));
     float* sx = sb + 4 * kMaxDim + 1 + 3;
-    uint32_t* spos = reinterpret_cast<uint32_t*>(sx + kPredWarps * 2 * kMaxDim);
+    uint32_t* spos = reinterpret_cast<uint32_t*>(sx + kPredWarps * 2 * kMaxDim * G);
     stage_weights(V, sW, sb);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* xs = sx + warp * 2 * kMaxDim;
-    float* hs = xs + kMaxDim;
+    float* xs = sx + warp * 2 * kMaxDim * G;
+    float* hs = xs + kMaxDim * G;
     uint32_t* pos_w = spos + warp * (64 + 128);
-    for (uint32_t qi = blockIdx.x * kPredWarps + warp; qi < nq; qi += gridDim.x * kPredWarps) {
-        const uint8_t* qrow = q + (size_t)qi * ix.row_bytes;
-        uint64_t khi, klo;
-        warp_keys_positions(ix, qrow, pos_w, khi, klo, lane);
-        const uint32_t s = (uint32_t)lane % 8;
-        const uint4 qv0 = s < (ix.row_bytes >> 4) ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
-        query_features(ix, qrow, qv0, pos_w, khi, klo, xs, pos_w + 64, lane);
-        const float y = mlp_warp_forward(V, sW, sW + V.in * V.h1, sW + V.in * V.h1 + V.h1 * V.h2,
-                                         sb, xs, hs, lane);
-        if (lane == 0) {
-            const float e = fminf(fmaxf(y + margin, -1.0f), 30.0f);
-            float pf = ceilf(exp2f(e));
-            uint32_t p = (uint32_t)pf;
-            p = p < p_lo ? p_lo : (p > p_hi ? p_hi : p);
-            p_out[qi] = p;
+    constexpr int kLanes = 32 / G;   // per query
+    const uint32_t c = (uint32_t)lane % kLanes, s = (uint32_t)lane % 8;
+    for (uint64_t q0 = ((uint64_t)blockIdx.x * kPredWarps + warp) * G; q0 < nq;
+         q0 += (uint64_t)gridDim.x * kPredWarps * G) {
+        const uint32_t n = (uint32_t)min((uint64_t)G, nq - q0);
+        uint64_t khi = 0, klo = 0;
+        if (c < ix.P.curves && (uint32_t)lane / kLanes < n) {
+            curve_key_call(q + (size_t)(q0 + lane / kLanes) * ix.row_bytes, ix.P, c, khi, klo);
+            const uint64_t off = ix.list_off[c];
+            pos_w[lane] = lower_bound_key(ix, c, off, (uint32_t)(ix.list_off[c + 1] - off), khi,
+                                          klo);
         }
         __syncwarp();
+        for (uint32_t g = 0; g < n; ++g) {
+            const uint8_t* qrow = q + (size_t)(q0 + g) * ix.row_bytes;
+            const uint4 qv0 =
+                s < (ix.row_bytes >> 4) ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
+            const int from = (int)(g * kLanes + c);
+            const uint64_t kh = __shfl_sync(0xffffffffu, khi, from);
+            const uint64_t kl = __shfl_sync(0xffffffffu, klo, from);
+            query_features(ix, qrow, qv0, pos_w + g * kLanes, kh, kl, xs + g, pos_w + 64, lane, G);
+        }
+        float y[G];
+        mlp_warp_forward<G>(V, sW, sW + V.in * V.h1, sW + V.in * V.h1 + V.h1 * V.h2, sb, xs, hs,
+                            lane, y);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (lane == g && g < n) {
+                const float e = fminf(fmaxf(y[g] + margin, -1.0f), 30.0f);
+                uint32_t p = (uint32_t)ceilf(exp2f(e));
+                p = p < p_lo ? p_lo : (p > p_hi ? p_hi : p);
+                p_out[q0 + g] = p;
+            }
+        __syncwarp();
     }
+}
+
+template <int G>
+cudaError_t go_predict(const IndexView& ix, const MlpView& V, const void* q, uint32_t nq,
+                       float margin, uint32_t p_lo, uint32_t p_hi, uint32_t* p_out, int sms,
+                       cudaStream_t s) {
+    const size_t smem = pred_smem(V, G);
+    const cudaError_t e =
+        cudaFuncSetAttribute(predict_depths_kernel<G>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const uint32_t per = kPredWarps * G;
+    const unsigned blocks =
+        std::min((uint32_t)(((uint64_t)nq + per - 1) / per), (uint32_t)sms * 8);
+    predict_depths_kernel<G><<<blocks, kPredWarps * 32, smem, s>>>(
+        ix, V, static_cast<const uint8_t*>(q), nq, margin, p_lo, p_hi, p_out);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- labels
@@ -980,19 +1086,20 @@ cudaError_t launch_predict_depths(hc_mlp* M, const hc_index* idx, const void* q,
     if (nq == 0) return cudaSuccess;
     if (refresh_bf16(M, s) != HC_OK) return cudaErrorUnknown;
     const MlpView V = view_of_mlp(M);
-    const size_t smem = pred_smem(V);
-    cudaError_t e = cudaFuncSetAttribute(predict_depths_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    unsigned blocks = (nq + kPredWarps - 1) / kPredWarps;
-    if (blocks > (unsigned)sms * 8) blocks = sms * 8;
-    predict_depths_kernel<<<blocks, kPredWarps * 32, smem, s>>>(
-        view_of(idx), V, static_cast<const uint8_t*>(q), nq, margin, p_lo, p_hi, p_out);
-    count_launches(1);
-    return cudaGetLastError();
+    const IndexView v = view_of(idx);
+    // Queries per warp: more where the warps in flight are full anyway (100,000
+    // queries, 8 curves: 854 us at one, 702 at two, 590 at four; 4,096: 65, 63, 70;
+    // 8,192: 107, 95, 104; 12,288: 143, 133, 123; 16 curves: 100,000 1,030 at one,
+    // 918 at two, but 12,288 176 and 183)
+    const uint32_t resident = (uint32_t)sms * 4 * kPredWarps;   // warps
+    if (v.P.curves <= 8 && nq >= 2 * resident)
+        return go_predict<4>(v, V, q, nq, margin, p_lo, p_hi, p_out, sms, s);
+    if (v.P.curves <= 16 && nq >= (v.P.curves <= 8 ? 1 : 6) * resident)
+        return go_predict<2>(v, V, q, nq, margin, p_lo, p_hi, p_out, sms, s);
+    return go_predict<1>(v, V, q, nq, margin, p_lo, p_hi, p_out, sms, s);
 }
 }  // namespace hc
 
