@@ -151,16 +151,6 @@ struct WarpTopK {
         }
     }
 
-    // a list that store() wrote earlier
-    __device__ __forceinline__ void load(uint32_t k, int lane, const int32_t* ids,
-                                         const uint32_t* dist) {
-#pragma unroll
-        for (int r = 0; r < KR; ++r) {
-            const uint32_t e = (uint32_t)r * 32 + lane;
-            v[r] = e < k && ids[e] >= 0 ? ((uint64_t)dist[e] << 32) | (uint32_t)ids[e] : kEmpty;
-        }
-    }
-
     // results e < k: ids (-1 for empty) and distances (empty -> int32 max or +inf)
     template <bool F32>
     __device__ __forceinline__ void store(uint32_t k, int lane, int32_t* ids, void* dist) const {

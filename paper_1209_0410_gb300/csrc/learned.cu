@@ -897,8 +897,8 @@ cudaError_t go_predict(const IndexView& ix, const MlpView& V, const void* q, uin
 // r 32 + lane in t[r] of the lane, and streams the ids of its windows past a
 // 2048-bit filter of them; the few ids that pass are compared with all: about
 // ten instructions per 32 ids, no row is read.  50,000 queries at p_max = 512 on
-// 10M rows and 8 lists: 8.1 ms, nearly all of it the one walk at p_max, against
-// 82.6 ms for a binary search over p (eleven walks).
+// 10M rows and 8 lists: 4.8 ms, nearly all of it the one walk at p_max, against
+// 82.4 ms for a binary search over p (eleven walks).
 constexpr int kLabelWarps = 8;
 constexpr uint32_t kLabelSlice = 1u << 17;   // queries labelled at once
 constexpr uint32_t kFilterBits = 2048;
