@@ -587,25 +587,40 @@ struct StagedSteps {
     const uint8_t* db;               // (values: a reference would put them in local memory)
     uint32_t row_bytes;
     uint8_t* ring;
-    uint4 q[8];                      // the query's vectors (zero past the row)
+    // the query's vectors (zero past the row) in registers, or, where a longer
+    // list leaves too few, read again for every step (80 registers, 60,000
+    // queries, k = 100, p = 16: 128-byte rows 1.68 against 1.73 ms with the vectors
+    // held; 96-byte rows at p = 200 4.6 against 5.2; 64-byte rows, k = 37, and
+    // k <= 32 are as fast or faster with them held)
+    static constexpr bool kHold = START || KR == 1 || (FULL && (KR == 2 || LPR < 8));
+    const uint8_t* qrow;
+    uint4 q[kHold ? 8 : 1];
     uint32_t id = 0, cnt = 0;        // of the step in flight (cnt = 0: none)
     uint32_t at = 0;                 // byte offset of its stage
     RowSwizzle sw;
     uint64_t thr;                    // the k-th candidate so far
     bool fresh;                      // no candidate so far
 
-    __device__ __forceinline__ StagedSteps(const IndexView& ix, const uint8_t* qrow,
+    __device__ __forceinline__ StagedSteps(const IndexView& ix, const uint8_t* query,
                                            uint8_t* ring_mem, const WarpTopK<KR>& top, uint32_t k)
         : db(static_cast<const uint8_t*>(ix.db)),
           row_bytes(ix.row_bytes),
           ring(ring_mem),
+          qrow(query),
           sw(ix.row_bytes >> 4),
           thr(top.kth(k)) {
         fresh = START && __all_sync(0xffffffffu, top.v[0] == kEmpty);
+        if constexpr (kHold)
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-            q[c] = c < LPR && (FULL || (uint32_t)c < (row_bytes >> 4)) ? ldg16(qrow + c * 16)
-                                                                       : make_uint4(0, 0, 0, 0);
+            for (int c = 0; c < 8; ++c)
+                q[c] = c < LPR && (FULL || (uint32_t)c < (row_bytes >> 4))
+                           ? ldg16(qrow + c * 16)
+                           : make_uint4(0, 0, 0, 0);
+    }
+
+    __device__ __forceinline__ uint4 query_vec(int c) const {
+        if constexpr (kHold) return q[c];
+        else return ldg16(qrow + c * 16);
     }
 
     __device__ __forceinline__ uint32_t other_stage() const {
@@ -659,7 +674,7 @@ struct StagedSteps {
             float part[LPR];
 #pragma unroll
             for (int c = 0; c < LPR; ++c)
-                part[c] = (uint32_t)c < vecs ? acc_vec(vec(c), q[c], 0.f) : 0.f;
+                part[c] = (uint32_t)c < vecs ? acc_vec(vec(c), query_vec(c), 0.f) : 0.f;
 #pragma unroll
             for (int w = LPR / 2; w >= 1; w >>= 1)
 #pragma unroll
@@ -669,7 +684,7 @@ struct StagedSteps {
             uint32_t acc[2] = {0, 0};
 #pragma unroll
             for (int c = 0; c < LPR; ++c)
-                if ((uint32_t)c < vecs) acc[c & 1] = acc_vec(vec(c), q[c], acc[c & 1]);
+                if ((uint32_t)c < vecs) acc[c & 1] = acc_vec(vec(c), query_vec(c), acc[c & 1]);
             return acc[0] + acc[1];
         }
     }
@@ -867,8 +882,14 @@ __device__ __forceinline__ void walk_wide(const IndexView& ix, const uint8_t* qr
 }
 
 // ring: kRingRows rows of the warp's shared memory (rows of at most 128 bytes) or
-// kWideRing bytes; SPLIT: steps part, part + parts, ... only; START as in StagedSteps
-template <bool F32, int LPR, int KR, bool SPLIT, bool START>
+// kWideRing bytes; SPLIT: steps part, part + parts, ... only; START as in
+// StagedSteps.  ROWS: kFullRows for rows of exactly 16 LPR bytes, kShortRows for
+// shorter ones, kAnyRows where one kernel serves both (a kernel of its own for
+// each spares registers: with both in one, 96-byte rows at k = 100 spilled, 5.2 against
+// 4.6 ms for 60,000 queries at p = 200).
+enum RowForm { kAnyRows, kFullRows, kShortRows };
+
+template <bool F32, int LPR, int KR, bool SPLIT, bool START, int ROWS = kAnyRows>
 __device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* qrow, uint32_t k,
                                             const uint32_t* win_at, const uint32_t* win_pre,
                                             uint32_t nm, uint32_t total, uint32_t part,
@@ -877,7 +898,7 @@ __device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* 
     if constexpr (LPR > 8) {
         walk_wide<F32, LPR, KR, SPLIT>(ix, qrow, k, win_at, win_pre, nm, total, part, parts, ring,
                                        top, lane);
-    } else if (ix.row_bytes == 16 * LPR) {
+    } else if (ROWS == kFullRows || (ROWS == kAnyRows && ix.row_bytes == 16 * LPR)) {
         walk_staged<F32, LPR, KR, true, SPLIT, START>(ix, qrow, k, win_at, win_pre, nm, total,
                                                       part, parts, ring, top, lane);
     } else {
@@ -889,7 +910,7 @@ __device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* 
 // Algorithm 2 for one query over the lists L0, L0 + Lstep, ... into the warp's
 // running top-k: positions, packed windows, then their walk.  pos_w, win_pre:
 // one word per list of the index.
-template <bool F32, int LPR, int KR, bool START = false>
+template <bool F32, int LPR, int KR, bool START = false, int ROWS = kAnyRows>
 __device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t* qrow,
                                              uint32_t depth, uint32_t k, uint32_t L0,
                                              uint32_t Lstep, uint32_t* pos_w, uint32_t* win_pre,
@@ -900,8 +921,8 @@ __device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t*
     const uint32_t nm = ix.lists > L0 ? (ix.lists - L0 + Lstep - 1) / Lstep : 0;
     uint32_t* win_at = pos_w;   // positions are consumed by pack_windows
     const uint32_t total = pack_windows(ix, depth, L0, Lstep, pos_w, win_at, win_pre, lane);
-    walk_packed<F32, LPR, KR, false, START>(ix, qrow, k, win_at, win_pre, nm, total, 0, 1, ring,
-                                            top, lane);
+    walk_packed<F32, LPR, KR, false, START, ROWS>(ix, qrow, k, win_at, win_pre, nm, total, 0, 1,
+                                                  ring, top, lane);
 }
 
 // The walk of a query's packed windows in the order of the row ids, kSweep

@@ -38,7 +38,7 @@ namespace {
 // Rows of at most 128 bytes go through a two-step cp.async ring in shared
 // memory: the block's rings, then its positions and window prefixes.
 // BLOCKS: blocks resident per SM (registers)
-template <bool F32, int LPR, int KR, int BLOCKS>
+template <bool F32, int LPR, int KR, int BLOCKS, int ROWS>
 __global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a
     uint32_t* pos_w = reinterpret_cast<uint32_t*>(smem + kQWarps * rb) + warp * 2 * ix.lists;
     WarpTopK<KR> top;
     top.init();
-    search_lists<F32, LPR, KR, BLOCKS == 2>(
+    search_lists<F32, LPR, KR, BLOCKS == 2, ROWS>(
         ix, qrow, depth, a.k, 0, 1, pos_w, pos_w + ix.lists, smem + warp * rb, top, lane,
         a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
         a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
@@ -256,49 +256,84 @@ struct QueryLaunch {
     static cudaError_t run(const QueryArgs& a, bool by_partition, cudaStream_t s) {
         const size_t smem =
             kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 2 * sizeof(uint32_t) * a.ix.lists);
-        if constexpr (LPR <= 8 && !F32)
-            if (by_partition) return go(query_kernel<F32, LPR, KR, 2>, a, smem, s);
-        return go(query_kernel<F32, LPR, KR, 3>, a, smem, s);
+        if constexpr (LPR <= 8) {
+            const bool full = a.ix.row_bytes == 16 * LPR;
+            if constexpr (!F32 && KR != 4)   // walk_kind: uint8, k <= 64
+                if (by_partition)
+                    return full ? go(query_kernel<F32, LPR, KR, 2, kFullRows>, a, smem, s)
+                                : go(query_kernel<F32, LPR, KR, 2, kShortRows>, a, smem, s);
+            return full ? go(query_kernel<F32, LPR, KR, 3, kFullRows>, a, smem, s)
+                        : go(query_kernel<F32, LPR, KR, 3, kShortRows>, a, smem, s);
+        } else {
+            return go(query_kernel<F32, LPR, KR, 3, kAnyRows>, a, smem, s);
+        }
     }
 };
 
+int sm_count() {
+    int sms = 152, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 // The address translation of an SM reaches 256 MB (128 pages of 2 MB: random
 // 128-byte rows of up to 256 MB arrive at 22 TB/s, of 384 MB at 8.4, of 1.2 GB at
-// 5.7, all of them in L2).  A batch in key order reads its rows of a larger
-// database
+// 5.7, all of them in L2).  A batch that fills the SMs several times over reads its
+// rows of a larger database
 //   kByPartition  when a partition's rows are within reach: the walk goes
 //                 partition by partition as it is, and with 16 instead of 24
 //                 warps per SM they stay in the same one (8 partitions of 160
-//                 MB, 100,000 queries at p = 32: 4.2 against 6.3 ms, sweeps 4.6);
-//   kSweeps       otherwise, sorted by row id (100,000 queries at p = 128 on 10M
-//                 rows: 2.5 against 3.9 ms; 20M 3.0 against 4.2, 50M 3.8 against
-//                 4.4; 3M rows, 384 MB: 2.4 against 2.7; 1.5M rows, 192 MB: 2.4
-//                 against 1.8, so the line lies between).
+//                 MB, 100,000 queries at p = 32: 4.2 against 6.3 ms, sweeps 4.6;
+//                 8 of 128 MB, 60,000 queries, by window entries E: in key order
+//                 E = 768 0.92 against 0.86, 2,048 1.50 against 1.58; in arrival
+//                 order E = 512 1.27 against 1.52, 3,200 3.5 against 4.1);
+//   kSweeps       in key order otherwise, sorted by row id (100,000 queries at p =
+//                 128 on 10M rows: 2.5 against 3.9 ms; 20M 3.0 against 4.2, 50M 3.8
+//                 against 4.4; 3M rows, 384 MB: 2.4 against 2.7; 1.5M rows, 192
+//                 MB: 2.4 against 1.8, so the line lies between; 96-byte rows,
+//                 which straddle lines, 384 MB: 1.41 against 1.32, 768 MB: 1.47
+//                 against 1.72).  The sort of a sweep wants whole sweeps (60,000
+//                 queries, 1 GB: E = 256 0.58 against 0.48 ms, 768 0.84 against
+//                 0.99, but on 384 MB 0.83 against 0.75) and a short list (k = 37,
+//                 E = 2,048: 2.6 against 2.4, 4,096 3.3 against 3.7; k = 100 is
+//                 no faster).
 // In arrival order the rows come from DRAM, which then binds (sweeps 4.6 against
-// 4.2 ms), and rows wider than 128 bytes need fewer translations per byte.
-constexpr uint64_t kReachBytes = 320ull << 20;
+// 4.2 ms), and rows wider than 128 bytes need fewer translations per byte.  3,000
+// queries, one wave: 0.23 ms by partition, 0.20 plain; 12,000 gain as 60,000 do.
+constexpr uint64_t kReachBytes = 320ull << 20, kReachStraddling = 512ull << 20;
+constexpr uint64_t kReachPartition = 200ull << 20;
 
 Walk walk_kind(const QueryArgs& a) {
     const IndexView& ix = a.ix;
     const uint64_t bytes = ix.rows * ix.row_bytes, parts = ix.lists / ix.P.curves;
-    if (!a.pos_cm || ix.P.dtype != HC_U8 || ix.row_bytes > 128 || bytes < kReachBytes)
+    const bool whole_lines = (ix.row_bytes & (ix.row_bytes - 1)) == 0;
+    if (ix.P.dtype != HC_U8 || ix.row_bytes > 128 || a.p_query ||
+        bytes < (whole_lines ? kReachBytes : kReachStraddling) ||
+        a.nq < 4ull * sm_count() * 2 * kQWarps)
         return kPlain;
-    if (parts > 1 && bytes / parts < (200ull << 20)) return kByPartition;
-    return ix.lists <= 96 ? kSweeps : kPlain;   // two blocks' shared memory per SM
+    const uint64_t entries = 2ull * a.p * ix.lists;   // of a query's windows
+    if (parts > 1 && bytes / parts < kReachPartition)
+        return entries >= (!a.pos_cm ? 512 : a.k <= 32 ? 2048 : 4096) && a.k <= 64 ? kByPartition
+                                                                                   : kPlain;
+    // at most 96 lists: two blocks' shared memory per SM
+    return a.pos_cm && ix.lists <= 96 && a.k <= 64 && entries >= (a.k <= 32 ? 1024 : 3200)
+               ? kSweeps
+               : kPlain;
 }
 
 // Warps per query when a batch in arrival order would leave SMs idle: as many as
 // one block of kSplitWarps warps per SM still holds (a second block waits for
-// the first: 1,500 queries at two warps each took 83 us where 2,000 at one take 77).
+// the first: 1,500 queries at two warps each took 83 us where 2,000 at one take
+// 77).  Two warps pay for their second search and merge only with some entries per
+// list (1,200 queries, 8 lists: 256 entries 45.3 against 44.3 us, 512 48.5 against
+// 49.9; 32 lists: 512 63 against 58, 1,024 73 and 73, 2,048 88 against 92).
 uint32_t split_warps(const QueryArgs& a) {
     if (a.order) return 1;
-    int sms = 152, dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t sms = sm_count();
     uint32_t wpq = 1;
-    while (wpq < (uint32_t)kSplitWarps && 
-           (uint64_t)a.nq * wpq * 2 <= (uint64_t)sms * kSplitWarps)
-        wpq *= 2;
+    while (wpq < (uint32_t)kSplitWarps && (uint64_t)a.nq * wpq * 2 <= sms * kSplitWarps) wpq *= 2;
+    if (wpq == 2 && !a.p_query && (a.p < 16 || 2ull * a.p * a.ix.lists < 384)) return 1;
     return wpq;
 }
 

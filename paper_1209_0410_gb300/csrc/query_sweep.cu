@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kQWarps * 32, 2) sweep_kernel(QueryArgs a, uin
 template <bool F32, int LPR, int KR>
 struct SweepLaunch {
     static cudaError_t run(const QueryArgs& a, cudaStream_t s) {
-        if constexpr (!F32 && LPR <= 8 && KR != 2) {
+        if constexpr (!F32 && LPR <= 8 && KR != 4) {
             const size_t smem = kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) +
                                            sizeof(uint32_t) * sweep_words(a.ix.lists));
             const cudaError_t e =
@@ -67,7 +67,7 @@ struct SweepLaunch {
             count_launches(1);
             return cudaGetLastError();
         } else {
-            return cudaErrorInvalidValue;   // uint8 rows of at most 128 bytes (walk_kind)
+            return cudaErrorInvalidValue;   // walk_kind: uint8 rows of at most 128 bytes, k <= 64
         }
     }
 };
@@ -76,7 +76,7 @@ struct SweepLaunch {
 
 cudaError_t launch_sweeps(const QueryArgs& a, cudaStream_t s) {
     return dispatch<SweepLaunch>(a.ix.P.dtype == HC_F32, lanes_per_row(a.ix.row_bytes),
-                                 a.k <= 32 ? 1 : 4, a, s);
+                                 regs_for_k(a.k), a, s);
 }
 
 }  // namespace hc

@@ -77,3 +77,26 @@ def test_large_databases_in_key_order(d, curves, m, parts, k, p, nq):
     idx = hc.hc_build(db, curves, m, partitions=parts)
     assert same(hc.hc_query_ordered(idx, q, k, p), hc.hc_query(idx, q, k, p))
     assert same(hc.hc_query_ordered(idx, q, k, 0), hc.hc_query(idx, q, k, 0))
+
+
+@pytest.mark.parametrize("mb,d,curves,m,parts,k,p,over", [
+    (350, 128, 8, 16, 1, 10, 64, 0), (350, 128, 8, 16, 1, 32, 67, 5),
+    (350, 128, 3, 16, 1, 1, 171, 1), (350, 128, 8, 16, 1, 33, 200, 3),
+    (350, 64, 4, 8, 1, 64, 401, 0), (350, 16, 1, 16, 1, 10, 512, 7),
+    (530, 112, 7, 16, 1, 10, 74, 9), (530, 48, 3, 16, 2, 17, 90, 1),
+    (450, 128, 8, 16, 2, 10, 32, 2), (350, 128, 8, 16, 2, 10, 64, 4),
+    (350, 64, 4, 16, 8, 40, 64, 1), (350, 128, 8, 16, 12, 10, 11, 6),
+    (350, 128, 8, 16, 2, 10, 16, 1), (350, 128, 8, 16, 1, 100, 70, 1)])
+def test_large_batches_of_large_databases(mb, d, curves, m, parts, k, p, over):
+    """Batches that fill the SMs several times: sweeps in key order, whole and cut
+    ones, and the walk partition by partition in both orders, at and past the lines
+    where they start, equal small batches."""
+    from paper_1209_0410_gb300 import hc
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nq = 4 * sms * 16 + over
+    db, q = make((mb << 20) // d + 13, d, "u8", nq, d + p)
+    idx = hc.hc_build(db, curves, m, partitions=parts)
+    small = [hc.hc_query(idx, q[a:a + 2500].contiguous(), k, p) for a in range(0, nq, 2500)]
+    want = [torch.cat([s[i] for s in small]) for i in (0, 1)]
+    assert same(hc.hc_query(idx, q, k, p), want)
+    assert same(hc.hc_query_ordered(idx, q, k, p), want)
