@@ -577,8 +577,9 @@ struct RowSwizzle {
 // next step's ids (lane l: row l; the rows of lanes at or past cnt are copied but
 // not offered), finish() reduces the last one.  ring: two stages of 32 rows,
 // 128-byte aligned.  START: the first step's candidates are sorted into the list
-// instead of inserted one by one (a call in the loop: where registers are short
-// its spills cost more than the insertions).
+// instead of inserted one by one (a call in the loop: with 80 registers its spills
+// cost more than the insertions for k > 32 and rows over 64 bytes; elsewhere it
+// gains 3-4% over all depths, 64-byte rows at k = 100 8%).
 constexpr uint32_t kRingRows = 64;     // two stages of 32 rows
 constexpr uint32_t kWideRing = 8192;   // bytes: two stages of walk_wide
 
@@ -587,12 +588,12 @@ struct StagedSteps {
     const uint8_t* db;               // (values: a reference would put them in local memory)
     uint32_t row_bytes;
     uint8_t* ring;
-    // the query's vectors (zero past the row) in registers, or, where a longer
-    // list leaves too few, read again for every step (80 registers, 60,000
-    // queries, k = 100, p = 16: 128-byte rows 1.68 against 1.73 ms with the vectors
-    // held; 96-byte rows at p = 200 4.6 against 5.2; 64-byte rows, k = 37, and
-    // k <= 32 are as fast or faster with them held)
-    static constexpr bool kHold = START || KR == 1 || (FULL && (KR == 2 || LPR < 8));
+    // the query's vectors (zero past the row) in registers, or, where they and the
+    // list (or the general row layout) do not fit beside each other, read again for
+    // every step (80 registers, 60,000 queries, k = 100, p = 16: 128-byte rows 1.68
+    // against 1.73 ms with the vectors held; 96-byte rows at p = 200 4.6 against 5.2;
+    // 64-byte rows and k = 37 are faster with them held)
+    static constexpr bool kHold = FULL && (START || KR <= 2 || LPR < 8);
     const uint8_t* qrow;
     uint4 q[kHold ? 8 : 1];
     uint32_t id = 0, cnt = 0;        // of the step in flight (cnt = 0: none)

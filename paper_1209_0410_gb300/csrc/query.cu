@@ -53,7 +53,8 @@ __global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a
     uint32_t* pos_w = reinterpret_cast<uint32_t*>(smem + kQWarps * rb) + warp * 2 * ix.lists;
     WarpTopK<KR> top;
     top.init();
-    search_lists<F32, LPR, KR, BLOCKS == 2, ROWS>(
+    constexpr bool kStart = LPR <= 8 && (BLOCKS == 2 || KR == 1 || LPR < 8);
+    search_lists<F32, LPR, KR, kStart, ROWS>(
         ix, qrow, depth, a.k, 0, 1, pos_w, pos_w + ix.lists, smem + warp * rb, top, lane,
         a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
         a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
