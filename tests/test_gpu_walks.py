@@ -70,8 +70,7 @@ def test_small_batches_equal_large(n, d, dtype, curves, m, parts, k, p, few):
     (112, 7, 16, 1, 10, 300, 99), (128, 8, 16, 2, 10, 40, 203), (64, 4, 16, 2, 100, 17, 203),
     (128, 8, 16, 12, 10, 9, 203), (128, 8, 16, 13, 10, 9, 203)])
 def test_large_databases_in_key_order(d, curves, m, parts, k, p, nq):
-    """350 MB of rows, above the reach of an SM's address translation: sweeps, whole
-    and cut ones, and the walk partition by partition."""
+    """350 MB of rows, above the reach of an SM's address translation, few queries."""
     from paper_1209_0410_gb300 import hc
     db, q = make((350 << 20) // d + 13, d, "u8", nq, d + p)
     idx = hc.hc_build(db, curves, m, partitions=parts)
