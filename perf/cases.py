@@ -232,21 +232,19 @@ def prepare(case, seed):
 
 # --------------------------------------------------------------------- a pass
 class _Lists:
-    """A device array of an index, as hc_index_describe gives its address; a tensor
-    made from it keeps the index alive."""
+    """A device array of an index, as hc_index_describe gives its address."""
 
-    def __init__(self, index, ptr, count, typestr):
-        self.index = index
+    def __init__(self, ptr, count, typestr):
         self.__cuda_array_interface__ = dict(shape=(count,), typestr=typestr, version=3,
                                              data=(ptr, False), strides=None)
 
 
 def _index_lists(index):
     info, off = hc.hc_index_describe(index)
-    out = [torch.as_tensor(_Lists(index, info["keys_hi_dev"], int(off[-1]), "<i8"), device=DEV),
-           torch.as_tensor(_Lists(index, info["ids_dev"], int(off[-1]), "<i4"), device=DEV)]
+    out = [torch.as_tensor(_Lists(info["keys_hi_dev"], int(off[-1]), "<i8"), device=DEV),
+           torch.as_tensor(_Lists(info["ids_dev"], int(off[-1]), "<i4"), device=DEV)]
     if info["keys_lo_dev"]:
-        out.append(torch.as_tensor(_Lists(index, info["keys_lo_dev"], int(off[-1]), "<i8"), device=DEV))
+        out.append(torch.as_tensor(_Lists(info["keys_lo_dev"], int(off[-1]), "<i8"), device=DEV))
     return out
 
 
