@@ -132,7 +132,7 @@ int check_params(const hc_build_params* p) {
     if (p->dims_per_curve < 1 || p->dims_per_curve > 16) return HC_ERR_ARG;
     if (p->bits != 8) return HC_ERR_ARG;
     const uint32_t parts = p->partitions ? p->partitions : 1;
-    if ((uint64_t)parts * p->curves > 256) return HC_ERR_ARG;
+    if ((uint64_t)parts * p->curves > kMaxLists) return HC_ERR_ARG;
     if ((uint64_t)p->curves * p->n >= (1ull << 32)) return HC_ERR_ARG;
     if (p->dim_map) {
         for (uint32_t i = 0; i < p->curves * p->dims_per_curve; ++i)

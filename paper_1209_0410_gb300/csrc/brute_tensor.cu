@@ -503,8 +503,7 @@ template <int ATOMS, int KS, int MT>
 cudaError_t launch_tensor(BruteArgs a, cudaStream_t s) {
     using S = BruteShape<ATOMS, KS, MT>;
     auto kernel = brute_tensor_kernel<ATOMS, KS, MT>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)S::kSmem);
+    cudaError_t e = allow_shared(kernel, S::kSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};

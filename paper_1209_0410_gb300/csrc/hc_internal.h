@@ -14,6 +14,18 @@ namespace hc {
 // Every kernel launch the library issues is counted here (hc_launch_count).
 void count_launches(uint64_t n);
 
+// Lists (partitions x curves) an index may have.
+constexpr uint32_t kMaxLists = 256;
+
+// Lets a kernel be launched with up to `most` bytes of dynamic shared memory.  The
+// limit belongs to the kernel, for every thread of the process, so `most` is the
+// largest need of any launch of it and never one launch's own: a smaller limit set
+// between another thread's call here and its launch would fail that launch.
+template <typename Kernel>
+cudaError_t allow_shared(Kernel* kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Host-side fault injection (hc_debug_fail_alloc): true when the library's
 // next allocation must report out-of-memory.
 bool alloc_should_fail();

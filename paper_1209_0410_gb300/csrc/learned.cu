@@ -469,9 +469,7 @@ __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __r
 // outputs into y, or with y null a training step's activations into M->work
 int launch_layers(hc_mlp* M, const float* x, const float* t, const uint32_t* perm, uint32_t n,
                   float* y, cudaStream_t s) {
-    if (cudaFuncSetAttribute(layers_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(LayerSmem)) != cudaSuccess)
-        return HC_ERR_CUDA;
+    if (allow_shared(layers_kernel, sizeof(LayerSmem)) != cudaSuccess) return HC_ERR_CUDA;
     const LayerArgs a{layout_of(M->in, M->h1, M->h2), M->params, M->in, M->h1, M->h2, n, x, t,
                       perm, y, work_of(M)};
     layers_kernel<<<tiles_of(n, kTile), 256, sizeof(LayerSmem), s>>>(a);
@@ -649,8 +647,8 @@ __global__ void __launch_bounds__(kPredWarps * 32) mlp_infer_kernel(MlpView V,
     }
 }
 
-size_t pred_smem(const MlpView& V, int G = 1) {
-    const uint32_t nw = V.in * V.h1 + V.h1 * V.h2 + V.h2;
+size_t pred_smem(uint32_t in, uint32_t h1, uint32_t h2, int G = 1) {
+    const uint32_t nw = in * h1 + h1 * h2 + h2;
     return ((nw * 2 + 15) & ~15u) + sizeof(float) * (4 * kMaxDim + 1 + 3) +
            sizeof(float) * kPredWarps * 2 * kMaxDim * G + sizeof(uint32_t) * kPredWarps * (64 + 128);
 }
@@ -874,10 +872,9 @@ template <int G>
 cudaError_t go_predict(const IndexView& ix, const MlpView& V, const void* q, uint32_t nq,
                        float margin, uint32_t p_lo, uint32_t p_hi, uint32_t* p_out, int sms,
                        cudaStream_t s) {
-    const size_t smem = pred_smem(V, G);
+    const size_t smem = pred_smem(V.in, V.h1, V.h2, G);
     const cudaError_t e =
-        cudaFuncSetAttribute(predict_depths_kernel<G>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_shared(predict_depths_kernel<G>, pred_smem(kMaxDim, kMaxDim, kMaxDim, G));
     if (e != cudaSuccess) return e;
     const uint32_t per = kPredWarps * G;
     const unsigned blocks =
@@ -1373,9 +1370,8 @@ HC_API int hc_mlp_forward(hc_mlp* M, const float* x_dev, uint32_t n, int bf16, f
     if (!bf16) return launch_layers(M, x_dev, nullptr, nullptr, n, y_dev, s);
     if (int rc = refresh_bf16(M, s)) return rc;
     const MlpView V = view_of_mlp(M);
-    const size_t smem = pred_smem(V);
-    if (cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+    const size_t smem = pred_smem(V.in, V.h1, V.h2);
+    if (allow_shared(mlp_infer_kernel, pred_smem(kMaxDim, kMaxDim, kMaxDim)) != cudaSuccess)
         return HC_ERR_CUDA;
     unsigned blocks = (n + kPredWarps - 1) / kPredWarps;
     if (blocks > 2048) blocks = 2048;

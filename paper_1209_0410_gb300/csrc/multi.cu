@@ -39,7 +39,6 @@ struct MultiTask {
 };
 
 constexpr int kMaxWarps = 16;
-constexpr uint32_t kMaxLists = 256;
 constexpr size_t kRingBytes = kWideRing;   // also kRingRows rows of at most 128 bytes
 static_assert(kRingBytes >= kRingRows * 128, "a ring for rows of either kind");
 
@@ -294,8 +293,7 @@ HC_API int hc_multi_plan_create(const hc_multi_job* jobs, uint32_t njobs,
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (const MultiJob& j : hj) P->lists_cap = std::max(P->lists_cap, (j.ix.lists + 3u) & ~3u);
     P->smem = multi_smem(cfg.warps_per_block, P->lists_cap);
-    if (cudaFuncSetAttribute(multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)P->smem) != cudaSuccess) {
+    if (allow_shared(multi_kernel, multi_smem(kMaxWarps, kMaxLists)) != cudaSuccess) {
         free_plan(P);
         return HC_ERR_CUDA;
     }

@@ -244,10 +244,12 @@ enum Walk { kPlain, kByPartition, kSweeps };
 
 template <bool F32, int LPR, int KR>
 struct QueryLaunch {
+    static size_t shared(uint32_t row_bytes, uint32_t lists) {
+        return kQWarps * (ring_bytes<LPR>(row_bytes) + 2 * sizeof(uint32_t) * lists);
+    }
     template <typename K>
     static cudaError_t go(K kernel, const QueryArgs& a, size_t smem, cudaStream_t s) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared(kernel, shared(16 * LPR, kMaxLists));
         if (e != cudaSuccess) return e;
         const unsigned blocks = (unsigned)(((uint64_t)a.nq + kQWarps - 1) / kQWarps);
         kernel<<<blocks, kQWarps * 32, smem, s>>>(a);
@@ -255,8 +257,7 @@ struct QueryLaunch {
         return cudaGetLastError();
     }
     static cudaError_t run(const QueryArgs& a, bool by_partition, cudaStream_t s) {
-        const size_t smem =
-            kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 2 * sizeof(uint32_t) * a.ix.lists);
+        const size_t smem = shared(a.ix.row_bytes, a.ix.lists);
         if constexpr (LPR <= 8) {
             const bool full = a.ix.row_bytes == 16 * LPR;
             if constexpr (!F32 && KR != 4)   // walk_kind: uint8, k <= 64

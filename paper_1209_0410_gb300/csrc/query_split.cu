@@ -64,16 +64,18 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 1) split_kernel(QueryArgs a,
 
 template <bool F32, int LPR, int KR>
 struct SplitLaunch {
+    // per: queries per block
+    static size_t shared(uint32_t row_bytes, uint32_t lists, uint32_t per) {
+        return kSplitWarps * (ring_bytes<LPR>(row_bytes) + 256 * KR + 4) + 8ull * per * lists;
+    }
     static cudaError_t run(const QueryArgs& a, uint32_t wpq, cudaStream_t s) {
         if constexpr (KR == 2) {
             return cudaErrorInvalidValue;   // launch_split takes 4
         } else {
-            const uint32_t per = kSplitWarps / wpq;   // queries per block
-            const size_t smem = kSplitWarps * (ring_bytes<LPR>(a.ix.row_bytes) + 256 * KR + 4) +
-                                8ull * per * a.ix.lists;
-            const cudaError_t e =
-                cudaFuncSetAttribute(split_kernel<F32, LPR, KR>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const uint32_t per = kSplitWarps / wpq;
+            const size_t smem = shared(a.ix.row_bytes, a.ix.lists, per);
+            const cudaError_t e = allow_shared(split_kernel<F32, LPR, KR>,
+                                               shared(16 * LPR, kMaxLists, kSplitWarps / 2));
             if (e != cudaSuccess) return e;
             split_kernel<F32, LPR, KR><<<(a.nq + per - 1) / per, kSplitWarps * 32, smem, s>>>(a, wpq);
             count_launches(1);

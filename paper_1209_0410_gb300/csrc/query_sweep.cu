@@ -52,13 +52,14 @@ __global__ void __launch_bounds__(kQWarps * 32, 2) sweep_kernel(QueryArgs a, uin
 
 template <bool F32, int LPR, int KR>
 struct SweepLaunch {
+    static size_t shared(uint32_t row_bytes, uint32_t lists) {
+        return kQWarps * (ring_bytes<LPR>(row_bytes) + sizeof(uint32_t) * sweep_words(lists));
+    }
     static cudaError_t run(const QueryArgs& a, cudaStream_t s) {
         if constexpr (!F32 && LPR <= 8 && KR != 4) {
-            const size_t smem = kQWarps * (ring_bytes<LPR>(a.ix.row_bytes) +
-                                           sizeof(uint32_t) * sweep_words(a.ix.lists));
+            const size_t smem = shared(a.ix.row_bytes, a.ix.lists);
             const cudaError_t e =
-                cudaFuncSetAttribute(sweep_kernel<F32, LPR, KR>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                allow_shared(sweep_kernel<F32, LPR, KR>, shared(16 * LPR, kMaxLists));
             if (e != cudaSuccess) return e;
             uint32_t shift = 0;
             while ((a.ix.rows - 1) >> shift > 255) ++shift;

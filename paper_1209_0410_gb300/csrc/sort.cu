@@ -1115,8 +1115,7 @@ int sort_body(const SortProblem& p, void* scratch, cudaStream_t s, bool& fenced)
     count_launches(1);
     if (cudaGetLastError() != cudaSuccess) return HC_ERR_CUDA;
     const size_t dyn_smem = sizeof(ScatterSmem);
-    e = cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dyn_smem);
+    e = allow_shared(scatter_kernel, dyn_smem);
     if (e != cudaSuccess) return HC_ERR_CUDA;
 
     const int digits = (int)((p.key_bits + 7) / 8);
