@@ -13,16 +13,19 @@ namespace {
 constexpr int kQWarps = 8;
 
 // Exact kNN: every row of the database, 32 rows per step, same distance and
-// top-k code as the query kernel.
+// top-k code as the query kernel.  again: only the queries whose output row the
+// kernel before marked kGaveUp.
 template <bool F32, int LPR, int KR>
 __global__ void __launch_bounds__(kQWarps * 32) brute_kernel(const uint8_t* __restrict__ db,
                                                             uint64_t n, uint32_t row_bytes,
                                                             const uint8_t* __restrict__ q,
                                                             uint32_t nq, uint32_t k,
-                                                            int32_t* out_ids, void* out_dist) {
+                                                            int32_t* out_ids, void* out_dist,
+                                                            bool again) {
+    if (again) asm volatile("griddepcontrol.wait;" ::: "memory");   // for the marks
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t qi = blockIdx.x * kQWarps + warp;
-    if (qi >= nq) return;
+    if (qi >= nq || (again && out_ids[(size_t)qi * k] != kGaveUp)) return;
     const uint8_t* qrow = q + (size_t)qi * row_bytes;
     const uint32_t s = (uint32_t)lane % LPR;
     const uint4 qv0 = s < (row_bytes >> 4) ? ldg16(qrow + s * 16) : make_uint4(0, 0, 0, 0);
@@ -43,12 +46,23 @@ __global__ void __launch_bounds__(kQWarps * 32) brute_kernel(const uint8_t* __re
 template <bool F32, int LPR, int KR>
 struct BruteLaunch {
     static cudaError_t run(const uint8_t* db, uint64_t n, uint32_t row_bytes, const uint8_t* q,
-                           uint32_t nq, uint32_t k, int32_t* ids, void* dist, cudaStream_t s) {
+                           uint32_t nq, uint32_t k, int32_t* ids, void* dist, bool again,
+                           cudaStream_t s) {
         const unsigned blocks = (nq + kQWarps - 1) / kQWarps;
-        brute_kernel<F32, LPR, KR><<<blocks, kQWarps * 32, 0, s>>>(db, n, row_bytes, q, nq, k,
-                                                                   ids, dist);
+        // the second look starts as the tensor-core kernel ends (2 us a call)
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(kQWarps * 32);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = again ? 1 : 0;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, brute_kernel<F32, LPR, KR>, db, n, row_bytes,
+                                                 q, nq, k, ids, dist, again);
         count_launches(1);
-        return cudaGetLastError();
+        return e == cudaSuccess ? cudaGetLastError() : e;
     }
 };
 
@@ -67,11 +81,17 @@ cudaError_t launch_bruteforce(const void* db, hc_dtype dtype, uint64_t n, uint32
                               void* out_dist, cudaStream_t s) {
     if (nq == 0) return cudaSuccess;
     const uint32_t row_bytes = dtype == HC_F32 ? d * 4 : d;
-    if (dtype == HC_U8 && n >= tensor_min_rows(k) && brute_tensor_takes(row_bytes, k))
-        return launch_brute_tensor(db, n, row_bytes, q, nq, k, out_ids, out_dist, s);
+    const bool tensor =
+        dtype == HC_U8 && n >= tensor_min_rows(k) && brute_tensor_takes(row_bytes, k);
+    if (tensor) {
+        const cudaError_t e = launch_brute_tensor(db, n, row_bytes, q, nq, k, out_ids, out_dist, s);
+        if (e != cudaSuccess) return e;
+    }
+    // all queries, or those the tensor cores gave up
     return dispatch<BruteLaunch>(dtype == HC_F32, lanes_per_row(row_bytes), regs_for_k(k),
                                  static_cast<const uint8_t*>(db), n, row_bytes,
-                                 static_cast<const uint8_t*>(q), nq, k, out_ids, out_dist, s);
+                                 static_cast<const uint8_t*>(q), nq, k, out_ids, out_dist, tensor,
+                                 s);
 }
 
 }  // namespace hc

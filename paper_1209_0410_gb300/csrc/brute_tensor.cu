@@ -12,7 +12,9 @@
 // share of the rows as B tiles of NB.  At the end the per-query lists of a
 // cluster's blocks meet in distributed shared memory, and each cluster merges its
 // lists into the output rows under a lock per row (the row's first id word), so
-// nothing is allocated and every SM has a share.  Warps:
+// nothing is allocated and every SM has a share.  A block in which a wait runs out
+// offers no list: its cluster marks its output rows kGaveUp, a mark that no merge
+// replaces, and launch_bruteforce searches marked rows again.  Warps:
 //   0 .. 4 MT - 1   epilogue, one query per thread (tensor-memory lane): the
 //                   scores against the query's threshold; the few that pass are
 //                   appended to the query's list in shared memory, which the
@@ -77,6 +79,14 @@ struct BruteArgs {
 };
 
 constexpr int32_t kLocked = -3;   // no id: ids are >= 0, -1 marks an empty slot
+
+// Looks at a barrier or a row lock before a role gives up.  (The tests build this
+// file with 0 and 1, so that waits run out; the wait for tensor-core work in flight
+// always has kWaitTries.)
+#ifndef HC_BRUTE_TRIES
+#define HC_BRUTE_TRIES kWaitTries
+#endif
+constexpr uint32_t kTries = HC_BRUTE_TRIES;
 
 // empty output rows, which the clusters then merge into
 __global__ void __launch_bounds__(256) empty_rows_kernel(uint64_t n, int32_t* ids, uint32_t* dist) {
@@ -171,6 +181,7 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     uint64_t* lists = reinterpret_cast<uint64_t*>(tailB + kBBufs * S::kBTail);
     uint64_t* bars = lists + (size_t)S::kQueries * KS;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4 * kBBufs);
+    volatile uint32_t* gave_up = tmem_slot + 1;   // a wait of this block ran out
     const uint32_t bar_full = smem_addr(bars);                 // B stage written
     const uint32_t bar_empty = bar_full + 8 * kBBufs;          // B stage consumed
     const uint32_t bar_done = bar_empty + 8 * kBBufs;          // accumulators complete
@@ -183,6 +194,7 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t tiles = (a.n + NB - 1) / NB;
     const uint64_t t0 = tiles * share / shares, t1 = tiles * (share + 1) / shares;
+    const uint32_t mytiles = (uint32_t)(t1 - t0);
     const uint32_t vecs = a.row_bytes >> 4;
 
     // A: twice the block's queries, and the constants of the |b|^2 digits (the
@@ -207,6 +219,7 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     for (uint32_t i = threadIdx.x; i < (uint32_t)(S::kQueries * KS); i += S::kThreads)
         lists[i] = kEmpty;
     if (threadIdx.x == 0) {
+        *gave_up = 0;
         for (int i = 0; i < kBBufs; ++i) {
             mbar_init(bar_full + 8 * i, kProducers / kBBufs);
             mbar_init(bar_empty + 8 * i, 1);
@@ -222,8 +235,8 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // A role that gives up on a wait ends its loop; the others then run out of
-    // their own bounded waits, and the block still reaches the barriers below.
+    // A role that gives up on a wait says so and ends its loop; the others then run
+    // out of their own bounded waits, and the block still reaches the barriers below.
     if (warp < 4 * MT) {
         // ------------------------------------------------ epilogue
         const uint32_t m = warp >> 2, ql = (uint32_t)warp * 32 + lane;   // query of the block
@@ -286,12 +299,13 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
                 tidy(__ballot_sync(0xffffffffu, pending == room));
             }
         };
-        for (uint64_t t = t0; t < t1; ++t) {
-            const uint32_t i = (uint32_t)(t - t0), buf = i % kBBufs, par = (i / kBBufs) & 1;
-            if (!mbar_wait_warp(bar_done + 8 * buf, par)) break;
+        uint32_t i = 0;   // row tile of the share
+        for (; i < mytiles; ++i) {
+            const uint32_t buf = i % kBBufs, par = (i / kBBufs) & 1;
+            if (!mbar_wait_warp(bar_done + 8 * buf, par, kTries)) break;
             tc_fence_after();
             const uint32_t acc = tmem + ((uint32_t)(warp & 3) << 21) + (buf * MT + m) * NB;
-            const uint32_t row0 = (uint32_t)(t * NB);
+            const uint32_t row0 = (uint32_t)(t0 + i) * NB;
             // the next 32 columns are on their way while these are looked over
             uint32_t d[2][32];
             tmem_ld32(acc, d[0]);
@@ -305,6 +319,7 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_drained + 8 * buf);
         }
+        if (i < mytiles) *gave_up = 1;
         __syncwarp();
         tidy(__ballot_sync(0xffffffffu, pending > 0));
     } else if (warp < 4 * MT + kProducers) {
@@ -332,7 +347,8 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
         };
         uint4 x[kPer], ahead[kPer];
         load(t0 + group, ahead);
-        for (uint64_t t = t0 + group; t < t1; t += kBBufs) {
+        uint64_t t = t0 + group;
+        for (; t < t1; t += kBBufs) {
             const uint32_t i = (uint32_t)(t - t0), buf = i % kBBufs, par = (i / kBBufs) & 1;
             int sq[kPer];
 #pragma unroll
@@ -360,7 +376,7 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
                     sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], o);
                 }
             }
-            if (!mbar_wait_warp(bar_empty + 8 * buf, par ^ 1)) break;
+            if (!mbar_wait_warp(bar_empty + 8 * buf, par ^ 1, kTries)) break;
             uint8_t* b = sB + buf * S::kBBytes;
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
@@ -380,13 +396,15 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_full + 8 * buf);
         }
+        if (t < t1) *gave_up = 1;
     } else if (lane == 0) {
         // ------------------------------------------------ MMA issue
         constexpr uint32_t idesc = mma_idesc_f16(128, NB);
-        for (uint64_t t = t0; t < t1; ++t) {
-            const uint32_t i = (uint32_t)(t - t0), buf = i % kBBufs, par = (i / kBBufs) & 1;
-            if (!mbar_wait(bar_drained + 8 * buf, par ^ 1)) break;
-            if (!mbar_wait(bar_full + 8 * buf, par)) break;
+        uint32_t issued = 0;   // row tiles of the share
+        for (; issued < mytiles; ++issued) {
+            const uint32_t buf = issued % kBBufs, par = (issued / kBBufs) & 1;
+            if (!mbar_wait(bar_drained + 8 * buf, par ^ 1, kTries)) break;
+            if (!mbar_wait(bar_full + 8 * buf, par, kTries)) break;
             tc_fence_after();
             const uint32_t b = smem_addr(sB) + buf * S::kBBytes;
             const uint64_t bt = mma_desc_plain(smem_addr(tailB) + buf * S::kBTail, NB * 16);
@@ -408,9 +426,10 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
             mma_commit(bar_done + 8 * buf);
         }
         // the tensor core is done with shared and tensor memory before they go
-        const uint32_t last = (uint32_t)(t1 - t0);
-        for (uint32_t i = last > kBBufs ? last - kBBufs : 0; i < last; ++i)
-            mbar_wait(bar_done + 8 * (i % kBBufs), (i / kBBufs) & 1);
+        bool whole = issued == mytiles;
+        for (uint32_t i = issued > kBBufs ? issued - kBBufs : 0; i < issued; ++i)
+            whole &= mbar_wait(bar_done + 8 * (i % kBBufs), (i / kBBufs) & 1, kWaitTries);
+        if (!whole) *gave_up = 1;
     }
     __syncwarp();
     tc_fence_before();
@@ -427,11 +446,18 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
     constexpr int KR = KS / 32, kWarps = S::kThreads / 32;
     const uint32_t turn = S::kQueries / blocks / kWarps * (share / blocks) / a.groups;
     const uint32_t rounds = (S::kQueries + blocks * kWarps - 1) / (blocks * kWarps);
+    bool whole = true;
+    for (uint32_t b = 0; b < blocks; ++b)
+        whole &= *cluster.map_shared_rank(tmem_slot + 1, b) == 0;
     for (uint32_t i = 0; i < rounds; ++i) {
         const uint32_t ql = rank + blocks * ((uint32_t)warp + kWarps * ((i + turn) % rounds));
         if (ql >= (uint32_t)S::kQueries || q0 + ql >= a.nq) continue;
         int32_t* ids = a.out_ids + (size_t)(q0 + ql) * a.k;
         uint32_t* dist = a.out_dist + (size_t)(q0 + ql) * a.k;
+        if (!whole) {
+            if (lane == 0) atomicExch(ids, kGaveUp);
+            continue;
+        }
         WarpTopK<KR> top;
         top.init();
         for (uint32_t b = 0; b < blocks; ++b) {
@@ -445,15 +471,16 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
             top.template store<false>(a.k, lane, ids, dist);
             continue;
         }
-        // take the row: its first id word says kLocked meanwhile
+        // take the row: its first id word says kLocked meanwhile (a holder lets go in
+        // microseconds); a mark found there, or left by giving up, is put back
         int32_t first = kLocked;
         if (lane == 0) {
-            const uint64_t t = global_ns();
-            do first = atomicExch(ids, kLocked);
-            while (first == kLocked && global_ns() - t < kMbarLimitNs);
+            for (uint32_t i = 0; i < kTries && first == kLocked; ++i)
+                first = atomicExch(ids, kLocked);
+            if (first == kLocked || first == kGaveUp) first = kGaveUp, atomicExch(ids, kGaveUp);
         }
         first = __shfl_sync(0xffffffffu, first, 0);
-        if (first == kLocked) continue;   // never: a holder lets go in microseconds
+        if (first == kGaveUp) continue;
         __threadfence();
 #pragma unroll
         for (int r = 0; r < KR; ++r) {
@@ -474,7 +501,9 @@ __global__ void __launch_bounds__(BruteShape<ATOMS, KS, MT>::kThreads, 1)
         }
         __threadfence();
         __syncwarp();
-        if (lane == 0) atomicExch(ids, top.v[0] == kEmpty ? -1 : (int32_t)(uint32_t)top.v[0]);
+        // let go, unless the row was marked meanwhile
+        if (lane == 0)
+            atomicCAS(ids, kLocked, top.v[0] == kEmpty ? -1 : (int32_t)(uint32_t)top.v[0]);
     }
     cluster.sync();
 }

@@ -192,7 +192,9 @@ cudaError_t launch_bruteforce(const void* db, hc_dtype dtype, uint64_t n, uint32
                               const void* q, uint32_t nq, uint32_t k, int32_t* out_ids,
                               void* out_dist, cudaStream_t s);
 // launch_bruteforce of uint8 rows on the tensor cores, for the widths and list
-// lengths brute_tensor_takes names
+// lengths brute_tensor_takes names.  An output row whose first id is kGaveUp (a wait
+// of the kernel ran out) is to be searched again.
+constexpr int32_t kGaveUp = -4;
 bool brute_tensor_takes(uint32_t row_bytes, uint32_t k);
 cudaError_t launch_brute_tensor(const void* db, uint64_t n, uint32_t row_bytes, const void* q,
                                 uint32_t nq, uint32_t k, int32_t* out_ids, void* out_dist,

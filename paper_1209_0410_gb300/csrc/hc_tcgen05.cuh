@@ -18,36 +18,32 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Waits for the phase of the given parity to complete; false when it has not
-// within kMbarLimitNs, so that no wait is endless (a wait of these kernels
-// lasts microseconds).
-constexpr uint64_t kMbarLimitNs = 2000000000ull;
-__device__ __forceinline__ uint64_t global_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
+// Waits for the phase of the given parity to complete; false when it has not after
+// `tries` looks of up to 2 us each, so that no wait is endless (a wait of these
+// kernels lasts microseconds).  Looks are counted instead of nanoseconds: time in
+// which the whole context does not run is no sign of a lost arrival.  (The time limit
+// in the instruction keeps the waiting warps from polling: without one, the search of
+// 2,000 queries on 10M rows takes 5.7 ms instead of 5.0.)
+constexpr uint32_t kWaitTries = 1u << 22;
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared.b64 p, [%1], %2, 2000;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
     return done != 0;
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    if (mbar_try(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (global_ns() - t0 < kMbarLimitNs)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t tries) {
+    for (uint32_t i = 0; i < tries; ++i)
         if (mbar_try(bar, parity)) return true;
     return false;
 }
 // the same for a whole warp, converged afterwards
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint32_t tries) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, tries));
 }
 
 // generic-proxy writes to shared memory made visible to the tensor core
