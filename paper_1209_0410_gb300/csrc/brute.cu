@@ -78,11 +78,27 @@ struct BruteLaunch {
 
 // Rows from which uint8 rows go to the tensor cores.  Below, every query still
 // meets many rows that enter its list, and there one warp per query (here)
-// beats one warp for 32 queries (there): 2,000 queries, k = 10: 79 against
-// 100 us at 2,048 rows, 148 against 118 us at 4,096; k = 100: 740 against 945 us
-// at 16,384 rows, from which on the time here grows with the rows and there
-// with their logarithm.
-constexpr uint64_t tensor_min_rows(uint32_t k) { return k <= 16 ? 4096 : 32768; }
+// beats one warp for 32 queries (there); from there on the time here grows with
+// the rows and there with their logarithm.  The line is lower where a row costs
+// more here, and higher where a list of 32 or 128 slots leaves less room for
+// rows not yet sorted in.  Times here / there, the lower of clustered and uniform
+// rows and of 33, 129 and 2,000 queries:
+//   rows <= 64 bytes   k = 1: 0.96 at 6,000 rows, 1.12 at 8,192; k = 5: 0.99 at 10,000, 1.13 at
+//                      12,288; k = 10: 0.60 at 4,096, 1.00 at 14,000; k = 16: 0.50 at 4,096,
+//                      0.99 at 20,000; k = 100: 0.74 at 32,768, 0.91 at 49,152, 1.07 at
+//                      65,536; k = 112: 0.51 at 32,768, 0.96 at 98,304, 1.17 at 131,072
+//   up to 128 bytes    k <= 10: 1.1 and more at 4,096; k = 16: 0.86 at 4,096, 1.03 at 6,000;
+//                      k = 112: 0.81 at 32,768, 1.02 at 49,152
+constexpr uint64_t tensor_min_rows(uint32_t row_bytes, uint32_t k) {
+    if (k <= 16) {
+        if (row_bytes <= 64) return 5500 + 950 * k;
+        return row_bytes <= 128 && k > 10 ? 6000 : 4096;
+    }
+    if (row_bytes > 128) return 32768;
+    // k <= 112 (brute_tensor_takes)
+    const uint64_t room = k < 128 ? 128 - k : 1, line = (row_bytes <= 64 ? 1650000 : 760000) / room;
+    return line > 32768 ? line : 32768;
+}
 
 }  // namespace
 
@@ -91,8 +107,8 @@ cudaError_t launch_bruteforce(const void* db, hc_dtype dtype, uint64_t n, uint32
                               void* out_dist, cudaStream_t s) {
     if (nq == 0) return cudaSuccess;
     const uint32_t row_bytes = dtype == HC_F32 ? d * 4 : d;
-    const bool tensor =
-        dtype == HC_U8 && n >= tensor_min_rows(k) && brute_tensor_takes(row_bytes, k);
+    const bool tensor = dtype == HC_U8 && n >= tensor_min_rows(row_bytes, k) &&
+                        brute_tensor_takes(row_bytes, k);
     if (tensor) {
         const cudaError_t e = launch_brute_tensor(db, n, row_bytes, q, nq, k, out_ids, out_dist, s);
         if (e != cudaSuccess) return e;
