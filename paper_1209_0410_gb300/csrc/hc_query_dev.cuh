@@ -366,13 +366,12 @@ __device__ __forceinline__ void query_positions(const IndexView& ix, const uint8
 // query_positions with the lanes of the warp spread over the searches: `each`
 // lanes (a power of two) take one list and probe `each` points of its bracket at
 // once, so a list of n entries takes log(n) / log(each + 1) rounds of one load
-// instead of log2(n).  For few lists per warp.
-__device__ __forceinline__ void query_positions_spread(const IndexView& ix, const uint8_t* qrow,
+// instead of log2(n).  For few lists per warp.  keys: the query's key (high, low)
+// on every curve.
+__device__ __forceinline__ void query_positions_spread(const IndexView& ix, const ulonglong2* keys,
                                                        uint32_t* pos_w, int lane, uint32_t L0,
                                                        uint32_t Lstep) {
     const uint32_t curves = ix.P.curves;
-    uint64_t khi = 0, klo = 0;
-    if ((uint32_t)lane < curves) curve_key_call(qrow, ix.P, (uint32_t)lane, khi, klo);
     const uint32_t mine = ix.lists > L0 ? (ix.lists - L0 + Lstep - 1) / Lstep : 0;
     uint32_t each = 32;
     while (each > 4 && 32 / each < mine) each /= 2;
@@ -382,8 +381,8 @@ __device__ __forceinline__ void query_positions_spread(const IndexView& ix, cons
         const uint32_t t = b + g;
         const bool on = t < mine;
         const uint32_t L = on ? L0 + t * Lstep : L0;
-        const uint64_t kh = __shfl_sync(0xffffffffu, khi, (int)(L % curves));
-        const uint64_t kl = __shfl_sync(0xffffffffu, klo, (int)(L % curves));
+        const ulonglong2 key = keys[L % curves];
+        const uint64_t kh = key.x, kl = key.y;
         const uint64_t off = ix.list_off[L], end = on ? ix.list_off[L + 1] : off;
         // first point in [first, first + count) where below() no longer holds
         auto search = [&](uint64_t first, uint64_t count, auto&& below) {

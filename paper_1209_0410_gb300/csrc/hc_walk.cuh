@@ -11,7 +11,8 @@
 namespace hc {
 
 constexpr int kQWarps = 8;       // warps per block, a query each
-constexpr int kSplitWarps = 16;  // warps per block that share queries
+constexpr int kSplitWarps = 16;  // warps that may share a query
+constexpr int kSplitBlock = 8;   // warps per block that share queries (16 for one query)
 
 struct QueryArgs {
     IndexView ix;

@@ -324,18 +324,31 @@ Walk walk_kind(const QueryArgs& a) {
                : kPlain;
 }
 
-// Warps per query when a batch in arrival order would leave SMs idle: as many as
-// one block of kSplitWarps warps per SM still holds (a second block waits for
-// the first: 1,500 queries at two warps each took 83 us where 2,000 at one take
-// 77).  Two warps pay for their second search and merge only with some entries per
-// list (1,200 queries, 8 lists: 256 entries 45.3 against 44.3 us, 512 48.5 against
-// 49.9; 32 lists: 512 63 against 58, 1,024 73 and 73, 2,048 88 against 92).
+// Warps per query when a batch in arrival order would leave SMs idle.
+// Two as long as 16 warps per SM hold them (1,500 queries at two warps each took 83 us
+// where 2,000 at one take 77), if the walk is worth a second search and a merge: 384
+// entries (k = 10, 1,000 queries: 30 against 33 us), with the slower inserts of k > 32
+// 4,096 (k = 33: 1,024 entries 91 against 72 us, 4,096 the same).
+// Four and eight cost the chip 9 and 22 ns more per query, which a lone batch does not
+// notice but batches on other streams do (16 streams, 400 queries each, p = 64: 26 ns
+// per query at four, 17 at two).  So they are for batches that leave most of the chip
+// free (6 warps per SM hold them; such a batch takes no longer than its launch by the
+// host), and for walks of 128 KB of rows per warp, where the cost is within 10% (304
+// queries of 25,600 rows each: 106 us at eight, 150 at four).
 uint32_t split_warps(const QueryArgs& a) {
     if (a.order) return 1;
     const uint64_t sms = sm_count();
     uint32_t wpq = 1;
-    while (wpq < (uint32_t)kSplitWarps && (uint64_t)a.nq * wpq * 2 <= sms * kSplitWarps) wpq *= 2;
-    if (wpq == 2 && !a.p_query && (a.p < 16 || 2ull * a.p * a.ix.lists < 384)) return 1;
+    // bytes of a query's rows (taken as few where every query has its own depth)
+    const uint64_t entries = std::min(2ull * a.p * a.ix.lists, 1ull * a.ix.rows * a.ix.P.curves);
+    const uint64_t bytes = a.p_query ? 0 : entries * a.ix.row_bytes;
+    while (wpq < (uint32_t)kSplitWarps) {
+        const uint32_t w = 2 * wpq;
+        const bool long_walks = w <= (uint32_t)kSplitBlock && bytes >= (uint64_t)w << 17;
+        if ((uint64_t)a.nq * w > sms * (wpq == 1 || long_walks ? 16 : 6)) break;
+        wpq = w;
+    }
+    if (wpq == 2 && !a.p_query && (a.p < 16 || entries < (a.k <= 32 ? 384 : 4096))) return 1;
     return wpq;
 }
 
