@@ -533,19 +533,18 @@ __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2b
 // accumulation in float32, inputs ascending.  Lane j computes hidden units j and
 // j + 32 of all G samples: a weight is read and widened once for them, and an
 // input of all of them is one load (G = 4: 13 instructions for 8 FMAs; one
-// sample and one unit at a time took 4 for each).
-template <int G>
-__device__ __forceinline__ void mlp_layer(const __nv_bfloat16* w, uint32_t in, uint32_t out,
+// sample and one unit at a time took 4 for each).  UNITS = 1: layers of at most 32
+// units (8 -> 8 for 4M samples: 1.08 ms with the second unit computed all the same,
+// 0.90 without).
+template <int G, int UNITS>
+__device__ __forceinline__ void mlp_units(const __nv_bfloat16* w, uint32_t in, uint32_t out,
                                           const float* xs, int lane, float (&acc)[2][G]) {
     const __nv_bfloat16* w0 = w + min((uint32_t)lane, out - 1);
     const __nv_bfloat16* w1 = w + min((uint32_t)lane + 32, out - 1);
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int g = 0; g < G; ++g) acc[u][g] = 0.f;
 #pragma unroll 4
     for (uint32_t i = 0; i < in; ++i) {
-        const float v0 = __bfloat162float(w0[i * out]), v1 = __bfloat162float(w1[i * out]);
+        const float v0 = __bfloat162float(w0[i * out]);
+        const float v1 = UNITS > 1 ? __bfloat162float(w1[i * out]) : 0.f;
         float x[G];
         if constexpr (G == 4)
             *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xs + 4 * i);
@@ -555,9 +554,22 @@ __device__ __forceinline__ void mlp_layer(const __nv_bfloat16* w, uint32_t in, u
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             acc[0][g] = fmaf(x[g], v0, acc[0][g]);
-            acc[1][g] = fmaf(x[g], v1, acc[1][g]);
+            if constexpr (UNITS > 1) acc[1][g] = fmaf(x[g], v1, acc[1][g]);
         }
     }
+}
+
+template <int G>
+__device__ __forceinline__ void mlp_layer(const __nv_bfloat16* w, uint32_t in, uint32_t out,
+                                          const float* xs, int lane, float (&acc)[2][G]) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int g = 0; g < G; ++g) acc[u][g] = 0.f;
+    if (out > 32)
+        mlp_units<G, 2>(w, in, out, xs, lane, acc);
+    else
+        mlp_units<G, 1>(w, in, out, xs, lane, acc);
 }
 
 template <int G>
