@@ -332,20 +332,22 @@ Walk walk_kind(const QueryArgs& a) {
 // Four and eight cost the chip 9 and 22 ns more per query, which a lone batch does not
 // notice but batches on other streams do (16 streams, 400 queries each, p = 64: 26 ns
 // per query at four, 17 at two).  So they are for batches that leave most of the chip
-// free (6 warps per SM hold them; such a batch takes no longer than its launch by the
-// host), and for walks of 128 KB of rows per warp, where the cost is within 10% (304
-// queries of 25,600 rows each: 106 us at eight, 150 at four).
+// free (6 to 8 warps per SM hold them; such a batch takes no longer than its launch by
+// the host), and for walks on which they cost no more than 10%: 1,024 uint8 rows per
+// warp (32 steps; 304 queries of 25,600 rows each: 106 us at eight, 150 at four; at half
+// the rows, 400 queries on 16 streams run at 0.8 of a warp per query) or 128 KB of float32
+// rows.
 uint32_t split_warps(const QueryArgs& a) {
     if (a.order) return 1;
     const uint64_t sms = sm_count();
     uint32_t wpq = 1;
-    // bytes of a query's rows (taken as few where every query has its own depth)
+    // rows of a query (taken as few where every query has its own depth)
     const uint64_t entries = std::min(2ull * a.p * a.ix.lists, 1ull * a.ix.rows * a.ix.P.curves);
-    const uint64_t bytes = a.p_query ? 0 : entries * a.ix.row_bytes;
+    const uint64_t worth = a.ix.P.dtype == HC_F32 ? (128u << 10) / a.ix.row_bytes : 1024;
     while (wpq < (uint32_t)kSplitWarps) {
         const uint32_t w = 2 * wpq;
-        const bool long_walks = w <= (uint32_t)kSplitBlock && bytes >= (uint64_t)w << 17;
-        if ((uint64_t)a.nq * w > sms * (wpq == 1 || long_walks ? 16 : 6)) break;
+        const bool far = !a.p_query && w <= (uint32_t)kSplitBlock && entries >= w * worth;
+        if ((uint64_t)a.nq * w > sms * (w == 2 || far ? 16 : (w == 8 ? 8 : 6))) break;
         wpq = w;
     }
     if (wpq == 2 && !a.p_query && (a.p < 16 || entries < (a.k <= 32 ? 384 : 4096))) return 1;
