@@ -703,11 +703,14 @@ struct StagedSteps {
         top.offer_row(d, id, live, k, thr, lane);
     }
 
+    // between: called while the copies of both steps are in flight
+    template <typename Between>
     __device__ __forceinline__ void add(uint32_t nid, uint32_t ncnt, WarpTopK<KR>& top, uint32_t k,
-                                        int lane) {
+                                        int lane, Between&& between) {
         __syncwarp();   // every lane is done with the stage before it is refilled
         issue(nid, other_stage(), lane);
         cp_async_commit();
+        between();
         if (cnt) {
             cp_async_wait<1>();
             reduce(top, k, lane);
@@ -724,8 +727,9 @@ struct StagedSteps {
 };
 
 // The walk of a query's packed windows (rows of at most 128 bytes): steps
-// part, part + parts, ... of 32 entries, the ids of the next two on their way.
-template <bool F32, int LPR, int KR, bool FULL, bool SPLIT, bool START>
+// part, part + parts, ... of 32 entries, the ids of the next two on their way: asked
+// for before the next step's rows or (LATE) behind them.
+template <bool F32, int LPR, int KR, bool FULL, bool SPLIT, bool START, bool LATE>
 __device__ __forceinline__ void walk_staged(const IndexView& ix, const uint8_t* qrow, uint32_t k,
                                             const uint32_t* win_at, const uint32_t* win_pre,
                                             uint32_t nm, uint32_t total, uint32_t my_part,
@@ -744,8 +748,11 @@ __device__ __forceinline__ void walk_staged(const IndexView& ix, const uint8_t* 
     };
     uint32_t id0 = id_of(part, e), id1 = id_of(part + parts, e + stride);
     for (uint32_t s = part; s < steps; s += parts) {
-        const uint32_t id2 = id_of(s + 2 * parts, e + 2 * stride);
-        pipe.add(id0, min(32u, total - 32 * s), top, k, lane);
+        uint32_t id2 = 0;
+        if constexpr (!LATE) id2 = id_of(s + 2 * parts, e + 2 * stride);
+        pipe.add(id0, min(32u, total - 32 * s), top, k, lane, [&] {
+            if constexpr (LATE) id2 = id_of(s + 2 * parts, e + 2 * stride);
+        });
         e += stride;
         id0 = id1;
         id1 = id2;
@@ -883,13 +890,14 @@ __device__ __forceinline__ void walk_wide(const IndexView& ix, const uint8_t* qr
 
 // ring: kRingRows rows of the warp's shared memory (rows of at most 128 bytes) or
 // kWideRing bytes; SPLIT: steps part, part + parts, ... only; START as in
-// StagedSteps.  ROWS: kFullRows for rows of exactly 16 LPR bytes, kShortRows for
+// StagedSteps, LATE as in walk_staged.  ROWS: kFullRows for rows of exactly 16 LPR bytes, kShortRows for
 // shorter ones, kAnyRows where one kernel serves both (a kernel of its own for
 // each spares registers: with both in one, 96-byte rows at k = 100 spilled, 5.2 against
 // 4.6 ms for 60,000 queries at p = 200).
 enum RowForm { kAnyRows, kFullRows, kShortRows };
 
-template <bool F32, int LPR, int KR, bool SPLIT, bool START, int ROWS = kAnyRows>
+template <bool F32, int LPR, int KR, bool SPLIT, bool START, int ROWS = kAnyRows,
+          bool LATE = false>
 __device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* qrow, uint32_t k,
                                             const uint32_t* win_at, const uint32_t* win_pre,
                                             uint32_t nm, uint32_t total, uint32_t part,
@@ -899,18 +907,18 @@ __device__ __forceinline__ void walk_packed(const IndexView& ix, const uint8_t* 
         walk_wide<F32, LPR, KR, SPLIT>(ix, qrow, k, win_at, win_pre, nm, total, part, parts, ring,
                                        top, lane);
     } else if (ROWS == kFullRows || (ROWS == kAnyRows && ix.row_bytes == 16 * LPR)) {
-        walk_staged<F32, LPR, KR, true, SPLIT, START>(ix, qrow, k, win_at, win_pre, nm, total,
-                                                      part, parts, ring, top, lane);
+        walk_staged<F32, LPR, KR, true, SPLIT, START, LATE>(ix, qrow, k, win_at, win_pre, nm, total,
+                                                            part, parts, ring, top, lane);
     } else {
-        walk_staged<F32, LPR, KR, false, SPLIT, START>(ix, qrow, k, win_at, win_pre, nm, total,
-                                                       part, parts, ring, top, lane);
+        walk_staged<F32, LPR, KR, false, SPLIT, START, LATE>(ix, qrow, k, win_at, win_pre, nm,
+                                                             total, part, parts, ring, top, lane);
     }
 }
 
 // Algorithm 2 for one query over the lists L0, L0 + Lstep, ... into the warp's
 // running top-k: positions, packed windows, then their walk.  pos_w, win_pre:
 // one word per list of the index.
-template <bool F32, int LPR, int KR, bool START = false, int ROWS = kAnyRows>
+template <bool F32, int LPR, int KR, bool START = false, int ROWS = kAnyRows, bool LATE = false>
 __device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t* qrow,
                                              uint32_t depth, uint32_t k, uint32_t L0,
                                              uint32_t Lstep, uint32_t* pos_w, uint32_t* win_pre,
@@ -921,8 +929,8 @@ __device__ __forceinline__ void search_lists(const IndexView& ix, const uint8_t*
     const uint32_t nm = ix.lists > L0 ? (ix.lists - L0 + Lstep - 1) / Lstep : 0;
     uint32_t* win_at = pos_w;   // positions are consumed by pack_windows
     const uint32_t total = pack_windows(ix, depth, L0, Lstep, pos_w, win_at, win_pre, lane);
-    walk_packed<F32, LPR, KR, false, START, ROWS>(ix, qrow, k, win_at, win_pre, nm, total, 0, 1,
-                                                  ring, top, lane);
+    walk_packed<F32, LPR, KR, false, START, ROWS, LATE>(ix, qrow, k, win_at, win_pre, nm, total, 0,
+                                                        1, ring, top, lane);
 }
 
 // The walk of a query's packed windows in the order of the row ids, kSweep
@@ -983,7 +991,7 @@ __device__ __forceinline__ void walk_sweeps(const IndexView& ix, const uint8_t* 
         __syncwarp();
         for (uint32_t o = 0; o < cnt; o += 32) {
             const uint32_t n = min(32u, cnt - o);
-            pipe.add(sorted[o + min((uint32_t)lane, n - 1)], n, top, k, lane);
+            pipe.add(sorted[o + min((uint32_t)lane, n - 1)], n, top, k, lane, [] {});
         }
     }
     pipe.finish(top, k, lane);

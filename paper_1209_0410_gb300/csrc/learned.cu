@@ -1018,10 +1018,10 @@ __global__ void fit_targets_kernel(const uint32_t* __restrict__ labels, uint32_t
 // Feature statistics: mean, then the unbiased standard deviation about it
 // (two passes, float64 sums); mu = mean, isd = 1 / max(sd, 1e-3).  A column's sum
 // is 256 strided partial sums (sample i in partial i % 256), added up 32 at a
-// time by a butterfly and then in order.  A block takes 32 partials of eight
-// columns (one 32-byte sector of a row): a lane per partial, a warp per column,
-// 16 loads in flight per lane; sums[c][g]: the sum of partials 32 g .. of
-// column c (pass 1: of x, pass 2: of (x - mean)^2).
+// time by a butterfly and then in order.  A block is one warp: 32 partials of one
+// column, a lane per partial, 16 loads in flight per lane (the other columns of a
+// 32-byte sector come from L2: blocks of one g run side by side); sums[c][g]: the sum
+// of partials 32 g .. of column c (pass 1: of x, pass 2: of (x - mean)^2).
 constexpr uint32_t kStatGroups = 8;   // of 32 partial sums
 __device__ __forceinline__ double stat_total(const double* s) {
     double t = 0.0;

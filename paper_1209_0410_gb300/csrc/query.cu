@@ -19,9 +19,9 @@
 //       reduced, so the bytes in flight are bounded by shared memory instead of
 //       registers, and each lane then reads a whole row (16-byte vectors laid
 //       out so that no two lanes of a quarter-warp meet in a bank): no partial
-//       sums cross lanes.  Wider rows are gathered into registers, LPR lanes to
-//       a row and eight 16-byte loads in flight per lane, and reduce-scattered
-//       over the LPR lanes.  uint8 distances use vabsdiffu4 + dp4a (exact in
+//       sums cross lanes.  Wider rows go through a ring of two 4 KB units, LPR
+//       lanes to a row and eight 16-byte vectors per lane and unit, and are
+//       reduce-scattered over the LPR lanes.  uint8 distances use vabsdiffu4 + dp4a (exact in
 //       32-bit integers), float32 use fma;
 //   K5/K6 the 32 packed (distance, id) candidates are offered to one running
 //       warp top-k for the whole query, which drops duplicate ids: the union
@@ -38,7 +38,7 @@ namespace {
 // Rows of at most 128 bytes go through a two-step cp.async ring in shared
 // memory: the block's rings, then its positions and window prefixes.
 // BLOCKS: blocks resident per SM (registers)
-template <bool F32, int LPR, int KR, int BLOCKS, int ROWS>
+template <bool F32, int LPR, int KR, int BLOCKS, int ROWS, bool LATE = false>
 __global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kQWarps * 32, BLOCKS) query_kernel(QueryArgs a
     WarpTopK<KR> top;
     top.init();
     constexpr bool kStart = LPR <= 8 && (BLOCKS == 2 || KR == 1 || LPR < 8);
-    search_lists<F32, LPR, KR, kStart, ROWS>(
+    search_lists<F32, LPR, KR, kStart, ROWS, LATE>(
         ix, qrow, depth, a.k, 0, 1, pos_w, pos_w + ix.lists, smem + warp * rb, top, lane,
         a.pos_in ? a.pos_in + (size_t)qi * ix.lists : nullptr,
         a.pos_cm ? a.pos_cm + (size_t)qi * ix.lists : nullptr);
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) fence_kernel(const uint64_t* __restrict__
 }
 
 // How a batch is walked (walk_kind).
-enum Walk { kPlain, kByPartition, kSweeps };
+enum Walk { kPlain, kLate, kByPartition, kSweeps };
 
 template <bool F32, int LPR, int KR>
 struct QueryLaunch {
@@ -256,12 +256,15 @@ struct QueryLaunch {
         count_launches(1);
         return cudaGetLastError();
     }
-    static cudaError_t run(const QueryArgs& a, bool by_partition, cudaStream_t s) {
+    static cudaError_t run(const QueryArgs& a, Walk walk, cudaStream_t s) {
         const size_t smem = shared(a.ix.row_bytes, a.ix.lists);
         if constexpr (LPR <= 8) {
             const bool full = a.ix.row_bytes == 16 * LPR;
+            if constexpr (!F32 && KR == 1)   // walk_kind: uint8, whole lines, k <= 32
+                if (walk == kLate)
+                    return go(query_kernel<F32, LPR, KR, 3, kFullRows, true>, a, smem, s);
             if constexpr (!F32 && KR != 4)   // walk_kind: uint8, k <= 64
-                if (by_partition)
+                if (walk == kByPartition)
                     return full ? go(query_kernel<F32, LPR, KR, 2, kFullRows>, a, smem, s)
                                 : go(query_kernel<F32, LPR, KR, 2, kShortRows>, a, smem, s);
             return full ? go(query_kernel<F32, LPR, KR, 3, kFullRows>, a, smem, s)
@@ -279,9 +282,9 @@ int sm_count() {
     return sms;
 }
 
-// The address translation of an SM reaches 256 MB (128 pages of 2 MB: random
-// 128-byte rows of up to 256 MB arrive at 22 TB/s, of 384 MB at 8.4, of 1.2 GB at
-// 5.7, all of them in L2).  A batch that fills the SMs several times over reads its
+// The address translation of an SM reaches 256 MB (128 pages of 2 MB: 16 MB of
+// random 128-byte rows, all in L2, arrive at 22 TB/s when they are spread over up to
+// 256 MB, at 8.4 over 384 MB and at 5.7 over 1.2 GB).  A batch that fills the SMs several times over reads its
 // rows of a larger database
 //   kByPartition  when a partition's rows are within reach: the walk goes
 //                 partition by partition as it is, and with 16 instead of 24
@@ -306,10 +309,29 @@ int sm_count() {
 constexpr uint64_t kReachBytes = 320ull << 20, kReachStraddling = 512ull << 20;
 constexpr uint64_t kReachPartition = 200ull << 20;
 
+// A batch whose last wave is nearly full (full_waves) is done when its slowest warp
+// is.  On rows at or past the reach, asking for the ids behind the next step's rows
+// makes every walk of such a batch up to 11% shorter (k = 10, p = 300, 340 MB: 3,300
+// queries 0.30 against 0.34 ms, 7,296 0.58 against 0.62); elsewhere asking before them is
+// faster (4,000 to 6,000 queries 0 to 3%, 18,000 up to 9%, 128 MB 5 to 12%, depths that
+// differ up to 11%).
+constexpr uint64_t kLateBytes = 240ull << 20;
+
+bool full_waves(uint64_t nq, uint64_t most) {
+    const uint64_t wave = 3ull * kQWarps * sm_count();   // warps resident
+    if (nq > most * wave) return false;
+    const uint64_t last = nq % wave == 0 ? wave : nq % wave;
+    return 100 * last >= (nq <= wave ? 66 : 80) * wave;
+}
+
 Walk walk_kind(const QueryArgs& a) {
     const IndexView& ix = a.ix;
     const uint64_t bytes = ix.rows * ix.row_bytes, parts = ix.lists / ix.P.curves;
     const bool whole_lines = (ix.row_bytes & (ix.row_bytes - 1)) == 0;
+    if (ix.P.dtype == HC_U8 && (ix.row_bytes == 64 || ix.row_bytes == 128) && !a.order &&
+        !a.p_query && a.k <= 32 && bytes / parts >= kLateBytes &&
+        full_waves(a.nq, bytes / parts < kReachBytes ? 5 : 3))
+        return kLate;
     if (ix.P.dtype != HC_U8 || ix.row_bytes > 128 || a.p_query ||
         bytes < (whole_lines ? kReachBytes : kReachStraddling) ||
         a.nq < 4ull * sm_count() * 2 * kQWarps)
@@ -367,7 +389,7 @@ cudaError_t launch_query(const IndexView& ix, const void* q, uint32_t nq, uint32
     const Walk walk = walk_kind(a);
     if (walk == kSweeps) return launch_sweeps(a, s);
     return dispatch<QueryLaunch>(ix.P.dtype == HC_F32, lanes_per_row(ix.row_bytes), regs_for_k(k),
-                                 a, walk == kByPartition, s);
+                                 a, walk, s);
 }
 
 cudaError_t launch_order_keys(const IndexView& ix, const void* q, uint32_t nq, uint32_t ncurves,
