@@ -2,7 +2,8 @@
 // queries occupies the chip and a single one does not wait on a serial walk.
 // Bound by latency: the launch, two rounds of dependent loads for the key, four
 // or five for the search, then 1/16 of the steps (100,000 rows, p = 128: one query
-// 21 us against 56 with one warp; 1,000 queries at p = 64: 36 against 46 us).
+// repeated 20 us against 56 with one warp, a query not seen before 76 against 110 with
+// the first touch of its lines; 1,000 queries at p = 64: 34 against 47 us).
 // Batches of other streams fill the time a block waits: three blocks of 8 warps fit
 // an SM beside each other.  Blocks of 16 with 128 registers, one per SM, left 320
 // batches of 400 queries on 16 streams at 4.8 ms (p = 64; 2.2 ms now, 2.1 with a warp
