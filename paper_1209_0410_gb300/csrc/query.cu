@@ -358,17 +358,17 @@ Walk walk_kind(const QueryArgs& a) {
 // the host), and for walks on which they cost no more than 10%: 1,024 uint8 rows per
 // warp (32 steps; 304 queries of 25,600 rows each: 106 us at eight, 150 at four; at half
 // the rows, 400 queries on 16 streams run at 0.8 of a warp per query) or 128 KB of float32
-// rows.
+// rows, or where each query has its own depth, so that the deepest sets the time (458
+// queries at depths the predictor chose: 81 us at four warps, 111 at two).
 uint32_t split_warps(const QueryArgs& a) {
     if (a.order) return 1;
     const uint64_t sms = sm_count();
     uint32_t wpq = 1;
-    // rows of a query (taken as few where every query has its own depth)
     const uint64_t entries = std::min(2ull * a.p * a.ix.lists, 1ull * a.ix.rows * a.ix.P.curves);
     const uint64_t worth = a.ix.P.dtype == HC_F32 ? (128u << 10) / a.ix.row_bytes : 1024;
     while (wpq < (uint32_t)kSplitWarps) {
         const uint32_t w = 2 * wpq;
-        const bool far = !a.p_query && w <= (uint32_t)kSplitBlock && entries >= w * worth;
+        const bool far = w <= (uint32_t)kSplitBlock && (a.p_query || entries >= w * worth);
         if ((uint64_t)a.nq * w > sms * (w == 2 || far ? 16 : (w == 8 ? 8 : 6))) break;
         wpq = w;
     }
